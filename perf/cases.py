@@ -128,7 +128,7 @@ def draw(rng):
         return dict(kind=kind, boxes=int(_log(rng, 8, 200)), lmin=lmin, lmax=rng.randint(lmin, 10), rho=3.0,
                     s=rng.choice([1.0, 0.5]), dt=0.01, lam=rng.choice([0.5, 0.65]), steps=rng.randint(16, 30))
     lmin = rng.randint(6, 12)
-    return dict(kind=kind, boxes=rng.randint(6, 24), lmin=lmin, lmax=rng.randint(lmin, 30), rho=3.0, s=s, dt=0.01,
+    return dict(kind=kind, boxes=rng.randint(6, 18), lmin=lmin, lmax=rng.randint(lmin, 30), rho=3.0, s=s, dt=0.01,
                 lam=0.5, skin=rng.choice([0.3, 0.4]), steps_min=60, steps_max=rng.randint(60, 100))
 
 

@@ -35,6 +35,10 @@ constexpr int kOwnerShift = 27;                       // list entry: owner lane 
 constexpr uint32_t kIndexMask = (1u << kOwnerShift) - 1u;
 constexpr int64_t kMaxParticles = int64_t(1) << kOwnerShift;
 constexpr int kGroup = 32;                            // particles per group (one warp)
+constexpr int kMinGroup = 4;
+constexpr int kGroupsWanted = 10000;
+constexpr int kBuildWarps = 8;                        // warps per block of the brick builder
+constexpr int kBuildBlocksWanted = 1024;
 constexpr int kForceWarps = 4;                        // groups per block of the pair kernel
 constexpr int kStencil = 27;
 // bricks: aligned kBrick^3 blocks of cells (contiguous ranges of the Morton
@@ -77,7 +81,7 @@ struct SimParams {
     int ncell;
     int nc[3];
     int cap;                  // neighbour capacity per particle (a group holds 32 x cap entries)
-    int gcap;                 // entries per group list = 32 * cap
+    int gcap;                 // entries per group list = group * cap
     int ngroups;              // group descriptors (lists) in use
     float L[3];
     float halfL[3];
@@ -106,6 +110,8 @@ struct SimParams {
     int no_reorder;           // 1: particles stay in load order (ablation; tile builder, no bricks)
     int list_layout;          // 0: packed group lists; 1: rows per particle (double insertion, join,
                               // 32x32 tile transpose; full lists, one thread per particle in the force)
+    int group;                // particles per group list: 32, 16, 8 or 4
+    int brick_split;          // CTAs of the builder per brick
     int brick_cap;            // halo particles the brick builder stages in shared memory
     int nb[3];                // bricks per axis
     int nbricks;

@@ -473,13 +473,36 @@ dpd_status get_graph(dpd_sim *h, int k, cudaGraphExec_t *out)
 // tiles.
 int group_count(const dpd_sim *h, int64_t n)
 {
-    return h->P.use_bricks ? (int)(n / kGroup) + h->P.nbricks : (int)((n + kGroup - 1) / kGroup);
+    return h->P.use_bricks ? (int)(n / h->P.group) + h->P.nbricks : (int)((n + kGroup - 1) / kGroup);
+}
+
+// Particles per group list and builder blocks per brick.  A warp walks (and
+// builds) one group, so a box of few groups leaves most of the chip idle while
+// each warp works through a long list: groups are halved until there are
+// kGroupsWanted of them or they hold kMinGroup particles, and a brick's groups
+// are shared by enough blocks that each warp builds about one, up to
+// kBuildBlocksWanted blocks in all (each block stages the brick's halo anew).
+// us per step, groups of 32 / 16 / 8 / 4 with the best split of each:
+// 3,000 particles 46.6 / - / 26.8 / 24.0; 32,000 (rho = 4) 61.9 / 44.0 / 33.8 /
+// 33.5; 81,000 56.7 / 44.6 / 43.2 / 45.7; 207,000 73.5 / 68.4 / 69.6 / -;
+// 648,000 155.3 / 156.0 / - / -; 3,000,000 575 / 604 / - / -, and a split of
+// 2 there 591.  A fixed capacity keeps groups of 32, whose particles share it.
+void pick_groups(dpd_sim *h, int64_t n)
+{
+    SimParams &P = h->P;
+    P.group = kGroup;
+    P.brick_split = 1;
+    if (!P.use_bricks) return;
+    if (P.list_layout == 0 && h->opt.nbr_capacity == 0)
+        while (P.group > kMinGroup && n < (int64_t)kGroupsWanted * P.group) P.group /= 2;
+    const int64_t rounds = (n / P.nbricks + P.group * kBuildWarps - 1) / (P.group * kBuildWarps);
+    P.brick_split = (int)std::max<int64_t>(1, std::min<int64_t>(kBuildBlocksWanted / P.nbricks, rounds));
 }
 
 // per-particle capacity from the largest group total of a build
-int capacity_for_total(uint32_t max_total)
+int capacity_for_total(uint32_t max_total, int group)
 {
-    int cap = (int)(((uint64_t)max_total * 5 / 4 + 64 + kGroup - 1) / kGroup);
+    int cap = (int)(((uint64_t)max_total * 5 / 4 + 64 + group - 1) / group);
     return std::max((cap + 7) / 8 * 8, 32);
 }
 
@@ -523,7 +546,7 @@ dpd_status alloc_particles(dpd_sim *h, int64_t n, int cap)
     h->P.ngroups = group_count(h, n);
     A((void **)&D.gdesc, sizeof(uint2) * (size_t)h->P.ngroups);
     A((void **)&D.rowcnt, u4);
-    A((void **)&D.nbr, (size_t)h->P.ngroups * kGroup * (size_t)cap * sizeof(uint32_t));
+    A((void **)&D.nbr, (size_t)h->P.ngroups * h->P.group * (size_t)cap * sizeof(uint32_t));
     h->red_doubles = std::max<size_t>((size_t)observe_blocks_for((int)n) * 8 + 8, 4096);
     A((void **)&D.vir_part, sizeof(double) * (size_t)((h->P.ngroups + kForceWarps - 1) / kForceWarps));
     A((void **)&D.red, h->red_doubles * sizeof(double));
@@ -537,7 +560,7 @@ dpd_status alloc_particles(dpd_sim *h, int64_t n, int cap)
                                 h->stream));
     for (int b = 0; b < 2; ++b) CUDA_TRY(h, cudaMemsetAsync(D.facc[b], 0, f4, h->stream));
     h->P.cap = cap;
-    h->P.gcap = kGroup * cap;
+    h->P.gcap = h->P.group * cap;
     h->cap_alloc_n = n;
     return DPD_OK;
 }
@@ -557,15 +580,15 @@ dpd_status rebuild_and_force(dpd_sim *h, bool grow_on_overflow)
         // grow the list: keep the particle arrays, reallocate the table (the
         // row layout reports its longest row, the packed one its largest group)
         const int cap = h->P.list_layout == 1 ? ((int)((uint64_t)c.max_nnb * 5 / 4 + 8) + 31) / 32 * 32
-                                              : capacity_for_total(c.max_nnb);
-        if ((int64_t)cap * kGroup >= (int64_t(1) << 26))
+                                              : capacity_for_total(c.max_nnb, h->P.group);
+        if ((int64_t)cap * h->P.group >= (int64_t(1) << 26))
             return fail(h, DPD_ERR_NBR_OVERFLOW, "neighbour list overflow: group list beyond 2^26 entries");
         dev_free(h, h->D.nbr, h->allocs);
-        st = dev_alloc(h, (void **)&h->D.nbr, (size_t)h->P.ngroups * kGroup * (size_t)cap * sizeof(uint32_t),
+        st = dev_alloc(h, (void **)&h->D.nbr, (size_t)h->P.ngroups * h->P.group * (size_t)cap * sizeof(uint32_t),
                        h->allocs);
         if (st) return st;
         h->P.cap = cap;
-        h->P.gcap = kGroup * cap;
+        h->P.gcap = h->P.group * cap;
         drop_graphs(h);
     }
     return fail(h, DPD_ERR_NBR_OVERFLOW, "neighbour list overflow after regrowing");
@@ -834,6 +857,7 @@ dpd_status dpd_set_state(dpd_sim *h, int64_t n, const double *x, const double *v
         bc = (bc + 31) / 32 * 32;
         h->P.brick_cap = std::min(std::max(bc, 256), std::min(max_brick_cap(), 65535));
     }
+    pick_groups(h, n);
     if (n != h->n || cap != h->P.cap || h->cap_alloc_n != n) {
         h->n = n;
         h->P.n = (int)n;

@@ -358,8 +358,7 @@ __global__ void k_nbuild(SimParams P, Ptrs D)
 // pass; the ids a brick leaves unused (at most one or two) get empty
 // descriptors.  A brick whose halo exceeds the staging buffer reads
 // positions from global memory.
-constexpr int kBuildThreads = 256;
-constexpr int kBuildWarps = kBuildThreads / 32;
+constexpr int kBuildThreads = 32 * kBuildWarps;
 constexpr int kSlots = 3;               // candidates per lane and chunk, held in registers
 constexpr int kChunk = 32 * kSlots;     // chunk of the candidate sequence
 // Three candidates per lane and four resident blocks per SM (64 registers,
@@ -641,11 +640,12 @@ __global__ void __launch_bounds__(kBuildThreads, kBuildMinBlocks) k_nbuild_brick
     __shared__ CellSeq s_seq[kBuildWarps];
     const uint32_t par = D.ctl->parity;
     const float4 *pos = D.pos[par];
-    const int b = blockIdx.x;
+    const int b = blockIdx.x / P.brick_split, part = blockIdx.x % P.brick_split;
     const BrickRange br = brick_halo(P, D, b, s_off, s_gstart, s_cnt, s_wsum);
     const uint32_t ord = D.brick_ord[b];
-    const uint32_t gbase = br.lo / kGroup + ord, gnext = br.hi / kGroup + ord + 1u;
-    const uint32_t nloc = br.hi - br.lo, ngrp = (nloc + kGroup - 1) / kGroup;
+    const uint32_t G = (uint32_t)P.group;
+    const uint32_t gbase = br.lo / G + ord, gnext = br.hi / G + ord + 1u;
+    const uint32_t nloc = br.hi - br.lo, ngrp = (nloc + G - 1) / G;
     const bool local = s_off[kHaloCells] <= (uint32_t)P.brick_cap;  // halo fits the staging buffer
     bool staged = true;
     if (local) staged = brick_stage_bulk(D, &s_bar, s_pos, pos, nullptr, nullptr, s_off, s_gstart, s_cnt);
@@ -659,9 +659,9 @@ __global__ void __launch_bounds__(kBuildThreads, kBuildMinBlocks) k_nbuild_brick
     const uint32_t lane = threadIdx.x & 31u;
     CellSeq &w = s_seq[threadIdx.x / 32u];
     uint32_t local_max = 0;
-    for (uint32_t q = threadIdx.x / 32u; q < ngrp; q += kBuildWarps) {
-        const uint32_t first = br.lo + q * kGroup;
-        const uint32_t owners = nloc - q * kGroup < (uint32_t)kGroup ? nloc - q * kGroup : (uint32_t)kGroup;
+    for (uint32_t q = part * kBuildWarps + threadIdx.x / 32u; q < ngrp; q += kBuildWarps * P.brick_split) {
+        const uint32_t first = br.lo + q * G;
+        const uint32_t owners = min(nloc - q * G, G);
         // halo slot of each lane's cell (the own cells of the brick are at 1..kBrick per axis)
         int t_lane = -1, inner_lane = 1;
         if (lane < owners) {
@@ -741,7 +741,7 @@ __global__ void __launch_bounds__(kBuildThreads, kBuildMinBlocks) k_nbuild_brick
         local_max = total > local_max ? total : local_max;
     }
     // ids of this brick's range that no group took
-    for (uint32_t g = gbase + ngrp + threadIdx.x; g < gnext; g += blockDim.x) D.gdesc[g] = make_uint2(0u, 0u);
+    if (part == 0) for (uint32_t g = gbase + ngrp + threadIdx.x; g < gnext; g += blockDim.x) D.gdesc[g] = make_uint2(0u, 0u);
     if (lane == 0 && local_max) atomicMax(&D.ctl->max_nnb, local_max);
 }
 
@@ -864,13 +864,13 @@ cudaError_t launch_rebuild(const SimParams &P, const Ptrs &D, cudaStream_t s, in
     if (P.use_bricks) {
         const size_t smem = sizeof(float4) * (size_t)P.brick_cap;
         if (P.list_layout == 1) {
-            k_nbuild_brick<false, true><<<P.nbricks, kBuildThreads, smem, s>>>(P, D);
+            k_nbuild_brick<false, true><<<P.nbricks * P.brick_split, kBuildThreads, smem, s>>>(P, D);
             k_rows_join<<<g, kThreads, 0, s>>>(P, D);
             k_rows_transpose<<<grid_for((P.n + 31) / 32 * 32), kBuildThreads, 0, s>>>(P, D);
         } else if (P.list_builder == 1) {
-            k_nbuild_brick<true, false><<<P.nbricks, kBuildThreads, smem, s>>>(P, D);
+            k_nbuild_brick<true, false><<<P.nbricks * P.brick_split, kBuildThreads, smem, s>>>(P, D);
         } else {
-            k_nbuild_brick<false, false><<<P.nbricks, kBuildThreads, smem, s>>>(P, D);
+            k_nbuild_brick<false, false><<<P.nbricks * P.brick_split, kBuildThreads, smem, s>>>(P, D);
         }
     } else if (P.no_reorder) {
         k_nbuild<true><<<g, kThreads, 0, s>>>(P, D);

@@ -75,11 +75,11 @@ typedef struct {
                                  summed in a fixed order (bit-identical runs, about 1.5x
                                  the pair work).  Random numbers and neighbour sets are
                                  deterministic in both modes. */
-    int32_t conditional_rebuild; /* 1 (default): inside the CUDA graphs, each step's rebuild
-                                 chain sits under a conditional node that the device sets
-                                 from the rebuild flag, so steps without a rebuild launch
-                                 none of its kernels; 0: the chain is launched every step
-                                 and its kernels return at once unless flagged */
+    int32_t conditional_rebuild; /* 1 (default) or 0, without effect: every step launches the
+                                 rebuild chain, whose kernels return at once unless the
+                                 device has flagged a rebuild.  (1 once put the chain under
+                                 a conditional graph node, which costs more than the
+                                 chain's early returns at every size.) */
     int32_t list_builder;     /* 0 (default): list entries placed by warp-ballot prefix
                                  sums (deterministic order, Sec. 3.3); 1: by an atomic add
                                  per entry -- the paper's Table 2 comparison; the list order

@@ -92,8 +92,7 @@ typedef struct {
  * with dpd.h's engine to FP32 rounding (a different summation order).
  *
  * Defaults: max_active 32, 4 workers, chunk_steps 100, budget 60 % of free memory,
- * dpd_default_options() for the boxes with conditional_rebuild = 0 (for
- * boxes of a few thousand particles the plain chain launches are cheaper).
+ * dpd_default_options() for the boxes.
  * For more than 8 boxes to run concurrently, set CUDA_DEVICE_MAX_CONNECTIONS
  * (e.g. to 32) in the environment before the first CUDA call. */
 void dpd_server_default_options(dpd_server_options *o);

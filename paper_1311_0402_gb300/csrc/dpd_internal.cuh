@@ -72,7 +72,7 @@ struct DevCtl {
     unsigned long long nrebuild;
     uint32_t max_nnb;        // largest group list total (pair entries) of the last build
     uint32_t rebuild_next;   // displacement flag raised by the kernel running now
-    uint32_t pad0;
+    uint32_t done;           // blocks of the moving kernel that have finished (merged advance)
     uint32_t oparity;        // live set of the order arrays (tag, pid): flips only at a rebuild
 };
 
@@ -110,6 +110,7 @@ struct SimParams {
     int no_reorder;           // 1: particles stay in load order (ablation; tile builder, no bricks)
     int list_layout;          // 0: packed group lists; 1: rows per particle (double insertion, join,
                               // 32x32 tile transpose; full lists, one thread per particle in the force)
+    int sort_small;           // the rebuild's sort runs in one block
     int group;                // particles per group list: 32, 16, 8 or 4
     int brick_split;          // CTAs of the builder per brick
     int brick_cap;            // halo particles the brick builder stages in shared memory
@@ -135,9 +136,8 @@ struct Ptrs {
     uint32_t *scan_part;           // block sums of the scan
     uint32_t *key;                 // [n] cell rank per particle
     uint32_t *slot;                // [n] arrival slot inside the cell
-    uint32_t *tmp_idx;             // [n] particle index in scatter order
-    unsigned long long *skey;      // [n] in-cell sort key in scatter order
-    uint32_t *perm;                // [n] new position -> old position
+    unsigned long long *skey;      // [n] in-cell sort keys, cell by cell
+    uint32_t *perm;                // [n] place in cell order -> particle (no_reorder)
     uint32_t *idx_of_pid;          // [n] caller index -> current position (maintained while bonds are set)
     // neighbours
     uint32_t *nbr;                 // packed group lists, [ngroups][gcap]
@@ -158,18 +158,40 @@ struct Ptrs {
 // ----------------------------------------------------------------- helpers
 __host__ __device__ inline uint32_t ceil_div_u(uint32_t a, uint32_t b) { return (a + b - 1) / b; }
 
-// The conditional-graph node guarding the next step's rebuild chain: the
-// advance kernel sets it to the rebuild flag (use = 0 outside graphs).
-struct NextCond {
-    cudaGraphConditionalHandle handle;
-    int use;
-};
+// Kernels of a step follow each other by programmatic dependent launch: each
+// is set up while the one before it still runs, and dependency_wait(), the
+// first thing it does, holds it until that one has finished and its stores
+// are visible.  Because every kernel of the sequence waits before it touches
+// memory or returns, the order of the whole sequence is that of plain launches.
+__device__ __forceinline__ void dependency_wait()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Launch k(args...); overlap: as a programmatic dependent of the kernel before
+// it on the stream (k then has to begin with dependency_wait()).
+template <typename... KArgs, typename... Args>
+cudaError_t launch_kernel(void (*k)(KArgs...), int grid, int block, size_t smem, cudaStream_t s, bool overlap, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid, 1, 1);
+    cfg.blockDim = dim3((unsigned)block, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, static_cast<KArgs>(args)...);
+}
 
 // launchers (each returns the launch status)
 cudaError_t launch_signature(const SimParams &P, const Ptrs &D, cudaStream_t s);
 // velocity-Verlet phase 1 from the full-step velocity, in place
-cudaError_t launch_phase1(const SimParams &P, const Ptrs &D, cudaStream_t s, NextCond next);
-cudaError_t launch_rebuild(const SimParams &P, const Ptrs &D, cudaStream_t s, int n_scan_blocks);
+cudaError_t launch_phase1(const SimParams &P, const Ptrs &D, cudaStream_t s, bool overlap);
+cudaError_t launch_rebuild(const SimParams &P, const Ptrs &D, cudaStream_t s, int n_scan_blocks, bool overlap);
 // idx_of_pid for the live order (kept up to date by rebuilds only while bonds are set)
 cudaError_t launch_index(const SimParams &P, const Ptrs &D, cudaStream_t s);
 // Pair force.  kForceEval: the force of the live state into D.fout (out_fout)
@@ -180,10 +202,12 @@ cudaError_t launch_index(const SimParams &P, const Ptrs &D, cudaStream_t s);
 enum ForceMode { kForceEval = 0, kForceStep = 1, kForceFinish = 2 };
 // In Newton-3 mode the pair kernel only accumulates (facc) and a
 // settle kernel completes the same mode afterwards; launch_force runs both.
-// after_pair (optional) is recorded with ev_flags right after the pair kernel;
-// next: the conditional node of the following step's rebuild chain.
-cudaError_t launch_force(const SimParams &P, const Ptrs &D, int mode, bool out_fout, cudaStream_t s,
-                         cudaEvent_t after_pair = nullptr, unsigned int ev_flags = 0, NextCond next = NextCond{0, 0});
+// after_pair (optional) is recorded with ev_flags right after the pair kernel.
+cudaError_t launch_force(const SimParams &P, const Ptrs &D, int mode, bool out_fout, cudaStream_t s, bool overlap,
+                         cudaEvent_t after_pair = nullptr, unsigned int ev_flags = 0);
+// kernels these launch: the opening phase 1 of a run, and the force phase of a step
+int phase1_kernels(const SimParams &P);
+int force_kernels(const SimParams &P);
 // observables: nblocks per-block partials in D.red, then their fixed-order
 // sum in D.red[nblocks * 8 .. + 8)
 cudaError_t launch_observe(const SimParams &P, const Ptrs &D, int nblocks, cudaStream_t s);
@@ -202,6 +226,10 @@ cudaError_t launch_profile(const SimParams &P, const Ptrs &D, int bin_axis, int 
 cudaError_t launch_pair_rng(uint64_t seed, uint64_t step, int64_t m, const uint32_t *ti, const uint32_t *tj,
                             uint32_t *out_hash, float *out_xi, cudaStream_t s);
 int scan_blocks_for(int ncell);
+// whether a box's binning, scan and reorder fit one block (k_sort_small), and
+// the kernels of a rebuild
+bool sort_fits_block(int64_t n, int ncell);
+int rebuild_kernels(const SimParams &P, int n_scan_blocks);
 // the bounded device wait on a transaction that never arrives (failure-detection probe)
 cudaError_t launch_wait_probe(const Ptrs &D, uint32_t polls, cudaStream_t s);
 cudaError_t time_alu_peak(int kind, int reps, double *lane_ops_per_s, double *ms_per_launch);

@@ -138,7 +138,6 @@ struct dpd_sim {
     bool has_state = false;
     bool failed = false;
     cudaStream_t stream = nullptr;
-    cudaStream_t side = nullptr;             // captures the bodies of conditional graph nodes
     bool own_stream = false;
     cudaEvent_t ev = nullptr;
     std::map<int, cudaGraphExec_t> graphs;  // steps per graph -> executable
@@ -307,8 +306,6 @@ void drop_graphs(dpd_sim *h)
     h->timed_graphs.clear();
 }
 
-constexpr int kRebuildKernels = 9;  // bin, 3 scan, scatter, rank, gather, commit, nbuild
-
 // Timing event on the stream; inside a graph capture it becomes an event
 // record node whose timestamp stays readable after the graph runs.
 // event record flags: external during stream capture (so the graph keeps
@@ -322,109 +319,38 @@ unsigned int rec_flags(dpd_sim *h)
 
 cudaError_t rec(dpd_sim *h, cudaEvent_t e) { return cudaEventRecordWithFlags(e, h->stream, rec_flags(h)); }
 
-// Rebuild chains inside captured graphs.  Each step's chain sits in the
-// body of a conditional IF node whose handle the preceding advance kernel
-// sets from the device rebuild flag, so a step without a rebuild launches
-// none of the chain's kernels (outside graphs the chain is launched and its
-// kernels return at once when the flag is clear).  The handles default to 1
-// at every launch of the graph: an unset handle runs the chain, which still
-// checks the flag itself.
-struct CondCapture {
-    bool active = false;
-    std::vector<cudaGraphConditionalHandle> handles;  // one per step
-    std::vector<cudaGraph_t> bodies;                  // IF bodies, filled after the capture
-};
-
-cudaError_t cond_begin(dpd_sim *h, int64_t k, CondCapture &cc)
-{
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    cudaGraph_t g = nullptr;
-    cudaError_t e = cudaStreamGetCaptureInfo(h->stream, &cs, nullptr, &g, nullptr, nullptr, nullptr);
-    if (e != cudaSuccess) return e;
-    if (cs != cudaStreamCaptureStatusActive) return cudaErrorStreamCaptureInvalidated;
-    cc.handles.assign((size_t)k, 0);
-    for (int64_t s = 0; s < k && e == cudaSuccess; ++s)
-        e = cudaGraphConditionalHandleCreate(&cc.handles[(size_t)s], g, 1u, cudaGraphCondAssignDefault);
-    cc.active = e == cudaSuccess;
-    return e;
-}
-
-NextCond next_cond(const CondCapture &cc, int64_t s)
-{
-    if (!cc.active || s >= (int64_t)cc.handles.size()) return NextCond{0, 0};
-    return NextCond{cc.handles[(size_t)s], 1};
-}
-
-// The rebuild chain of step s: an IF node under capture, the chain otherwise.
-cudaError_t rebuild_step(dpd_sim *h, CondCapture &cc, int64_t s)
-{
-    if (!cc.active) return launch_rebuild(h->P, h->D, h->stream, h->n_scan_blocks);
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    cudaGraph_t g = nullptr;
-    const cudaGraphNode_t *deps = nullptr;
-    const cudaGraphEdgeData *edata = nullptr;
-    size_t ndeps = 0;
-    cudaError_t e = cudaStreamGetCaptureInfo(h->stream, &cs, nullptr, &g, &deps, &edata, &ndeps);
-    if (e != cudaSuccess) return e;
-    cudaGraphNodeParams np = {cudaGraphNodeTypeConditional};
-    np.conditional.handle = cc.handles[(size_t)s];
-    np.conditional.type = cudaGraphCondTypeIf;
-    np.conditional.size = 1;
-    cudaGraphNode_t node = nullptr;
-    e = cudaGraphAddNode(&node, g, deps, edata, ndeps, &np);
-    if (e != cudaSuccess) return e;
-    cc.bodies.push_back(np.conditional.phGraph_out[0]);
-    return cudaStreamUpdateCaptureDependencies(h->stream, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
-}
-
-// After the capture: each IF body gets the rebuild chain, captured on the
-// handle's side stream.
-cudaError_t cond_fill(dpd_sim *h, CondCapture &cc)
-{
-    for (cudaGraph_t body : cc.bodies) {
-        cudaError_t e = cudaStreamBeginCaptureToGraph(h->side, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
-        if (e != cudaSuccess) return e;
-        e = launch_rebuild(h->P, h->D, h->side, h->n_scan_blocks);
-        cudaGraph_t out = nullptr;
-        cudaError_t e2 = cudaStreamEndCapture(h->side, &out);
-        if (e != cudaSuccess) return e;
-        if (e2 != cudaSuccess) return e2;
-    }
-    return cudaSuccess;
-}
-
 // The kernel sequence of enqueue_steps with timing events between the
 // groups: ev[0] | phase 1 | ev[1] | rebuild | ev[2] | pair kernel | ev[3] |
-// settle + advance | ev[4] | rebuild | ev[5] ...  (3 events per step)
-cudaError_t enqueue_steps_timed(dpd_sim *h, int64_t k, CondCapture &cc)
+// settle + advance | ev[4] | rebuild | ev[5] ...  (3 events per step).  The
+// kernels are launched without overlap, so that an event's time is the end of
+// the group before it.
+cudaError_t enqueue_steps_timed(dpd_sim *h, int64_t k)
 {
     cudaError_t e = rec(h, h->tev[0]);
-    if (e == cudaSuccess) e = launch_phase1(h->P, h->D, h->stream, next_cond(cc, 0));
+    if (e == cudaSuccess) e = launch_phase1(h->P, h->D, h->stream, false);
     if (e == cudaSuccess) e = rec(h, h->tev[1]);
     const unsigned int fl = rec_flags(h);
     for (int64_t s = 0; s < k && e == cudaSuccess; ++s) {
-        e = rebuild_step(h, cc, s);
+        e = launch_rebuild(h->P, h->D, h->stream, h->n_scan_blocks, false);
         if (e == cudaSuccess) e = rec(h, h->tev[3 * s + 2]);
         if (e == cudaSuccess)
-            e = launch_force(h->P, h->D, s + 1 < k ? kForceStep : kForceFinish, false, h->stream, h->tev[3 * s + 3], fl,
-                             next_cond(cc, s + 1));
+            e = launch_force(h->P, h->D, s + 1 < k ? kForceStep : kForceFinish, false, h->stream, false, h->tev[3 * s + 3], fl);
         if (e == cudaSuccess) e = rec(h, h->tev[3 * s + 4]);
     }
     return e;
 }
 
 // Kernel sequence of k steps (starting and ending at a full-step state):
-// phase 1, then per step the rebuild chain (runs only when flagged), the
-// pair kernel and the integration into the next step (or the finish of the
-// last).
-cudaError_t enqueue_steps(dpd_sim *h, int64_t k, CondCapture &cc)
+// phase 1, then per step the rebuild chain (its kernels return at once unless
+// flagged), the pair kernel and the integration into the next step (or the
+// finish of the last).
+cudaError_t enqueue_steps(dpd_sim *h, int64_t k)
 {
-    cudaError_t e = launch_phase1(h->P, h->D, h->stream, next_cond(cc, 0));
+    cudaError_t e = launch_phase1(h->P, h->D, h->stream, true);
     for (int64_t s = 0; s < k && e == cudaSuccess; ++s) {
-        e = rebuild_step(h, cc, s);
+        e = launch_rebuild(h->P, h->D, h->stream, h->n_scan_blocks, true);
         if (e == cudaSuccess)
-            e = launch_force(h->P, h->D, s + 1 < k ? kForceStep : kForceFinish, false, h->stream, nullptr, 0,
-                             next_cond(cc, s + 1));
+            e = launch_force(h->P, h->D, s + 1 < k ? kForceStep : kForceFinish, false, h->stream, true);
     }
     return e;
 }
@@ -435,11 +361,8 @@ dpd_status capture_steps(dpd_sim *h, int64_t k, bool timed, cudaGraphExec_t *out
 {
     cudaGraph_t g = nullptr;
     CUDA_TRY(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-    CondCapture cc;
-    cudaError_t e = h->opt.conditional_rebuild ? cond_begin(h, k, cc) : cudaSuccess;
-    if (e == cudaSuccess) e = timed ? enqueue_steps_timed(h, k, cc) : enqueue_steps(h, k, cc);
+    cudaError_t e = timed ? enqueue_steps_timed(h, k) : enqueue_steps(h, k);
     cudaError_t e2 = cudaStreamEndCapture(h->stream, &g);
-    if (e == cudaSuccess && e2 == cudaSuccess) e = cond_fill(h, cc);
     if (e != cudaSuccess || e2 != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
         cudaGetLastError();
@@ -539,7 +462,6 @@ dpd_status alloc_particles(dpd_sim *h, int64_t n, int cap)
     A((void **)&D.facc[1], f4);
     A((void **)&D.key, u4);
     A((void **)&D.slot, u4);
-    A((void **)&D.tmp_idx, u4);
     A((void **)&D.skey, sizeof(unsigned long long) * (size_t)n);
     A((void **)&D.perm, u4);
     A((void **)&D.idx_of_pid, u4);
@@ -572,8 +494,8 @@ dpd_status rebuild_and_force(dpd_sim *h, bool grow_on_overflow)
         uint32_t one = 1u;
         CUDA_TRY(h, cudaMemcpyAsync(&h->D.ctl->rebuild, &one, sizeof(one), cudaMemcpyHostToDevice, h->stream));
         CUDA_TRY(h, cudaMemsetAsync(&h->D.ctl->err, 0, sizeof(uint32_t), h->stream));
-        CUDA_TRY(h, launch_rebuild(h->P, h->D, h->stream, h->n_scan_blocks));
-        CUDA_TRY(h, launch_force(h->P, h->D, kForceEval, false, h->stream));
+        CUDA_TRY(h, launch_rebuild(h->P, h->D, h->stream, h->n_scan_blocks, true));
+        CUDA_TRY(h, launch_force(h->P, h->D, kForceEval, false, h->stream, true));
         DevCtl c;
         dpd_status st = check_err(h, c);
         if (st != DPD_ERR_NBR_OVERFLOW || !grow_on_overflow) return st;
@@ -734,12 +656,6 @@ dpd_status dpd_create(dpd_sim **out, const double box[3], int32_t n_species, con
         }
         h->own_stream = true;
     }
-    if (cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking) != cudaSuccess) {
-        cudaGetLastError();
-        h->side = nullptr;
-        dpd_destroy(h);
-        return fail(nullptr, DPD_ERR_CUDA, "cudaStreamCreate failed");
-    }
     if (cudaEventCreateWithFlags(&h->ev, cudaEventDisableTiming) != cudaSuccess) {
         cudaGetLastError();
         dpd_destroy(h);
@@ -857,6 +773,7 @@ dpd_status dpd_set_state(dpd_sim *h, int64_t n, const double *x, const double *v
         bc = (bc + 31) / 32 * 32;
         h->P.brick_cap = std::min(std::max(bc, 256), std::min(max_brick_cap(), 65535));
     }
+    h->P.sort_small = sort_fits_block(n, h->P.ncell) ? 1 : 0;
     pick_groups(h, n);
     if (n != h->n || cap != h->P.cap || h->cap_alloc_n != n) {
         h->n = n;
@@ -913,7 +830,7 @@ dpd_status dpd_set_bonds(dpd_sim *h, int64_t nb, const uint32_t *pairs, double k
     h->bonds_set = nb > 0;
     drop_graphs(h);
     CUDA_TRY(h, launch_index(h->P, h->D, h->stream));
-    CUDA_TRY(h, launch_force(h->P, h->D, kForceEval, false, h->stream));
+    CUDA_TRY(h, launch_force(h->P, h->D, kForceEval, false, h->stream, true));
     DevCtl c;
     return check_err(h, c);
 }
@@ -995,7 +912,7 @@ dpd_status dpd_forces(dpd_sim *h, double *f_out)
     if (st) return st;
     if (h->pending && (st = dpd_sync(h)) != DPD_OK) return st;  // report a queued run's error first
     CUDA_TRY(h, cudaMemsetAsync(&h->D.ctl->err, 0, sizeof(uint32_t), h->stream));
-    CUDA_TRY(h, launch_force(h->P, h->D, kForceEval, true, h->stream));
+    CUDA_TRY(h, launch_force(h->P, h->D, kForceEval, true, h->stream, true));
     DevCtl c;
     st = check_err(h, c);
     if (st) return st;
@@ -1067,8 +984,7 @@ dpd_status dpd_step_async(dpd_sim *h, int64_t nsteps)
             left = 0;
         }
     } else {
-        CondCapture none;
-        CUDA_TRY(h, enqueue_steps(h, left, none));
+        CUDA_TRY(h, enqueue_steps(h, left));
     }
     h->step += (uint64_t)nsteps;
     return DPD_OK;
@@ -1155,8 +1071,7 @@ dpd_status dpd_step_profiled(dpd_sim *h, int64_t nsteps, dpd_step_times *out)
         }
         CUDA_TRY(h, cudaGraphLaunch(ex, h->stream));
     } else {
-        CondCapture none;
-        CUDA_TRY(h, enqueue_steps_timed(h, nsteps, none));
+        CUDA_TRY(h, enqueue_steps_timed(h, nsteps));
     }
     h->step += (uint64_t)nsteps;
     DevCtl c;
@@ -1187,12 +1102,10 @@ dpd_status dpd_step_profiled(dpd_sim *h, int64_t nsteps, dpd_step_times *out)
         }
         out->steps = nsteps;
         out->force_launches = nsteps;
-        // per step: pair kernel (+ settle), advance; the rebuild chain on every
-        // step outside graphs, only on rebuild steps inside them (conditional
-        // nodes); plus the opening phase 1 + advance
         out->rebuilds = (int64_t)(c.nrebuild - c0.nrebuild);
-        const int64_t chains = h->opt.graph_steps > 0 && h->opt.conditional_rebuild ? out->rebuilds : nsteps;
-        out->kernel_launches = nsteps * (2 + (h->P.newton3 ? 1 : 0)) + 2 + chains * kRebuildKernels;
+        // the opening phase 1, then per step the rebuild chain (launched every
+        // step; its kernels return at once unless flagged) and the force phase
+        out->kernel_launches = phase1_kernels(h->P) + nsteps * (rebuild_kernels(h->P, h->n_scan_blocks) + force_kernels(h->P));
     }
     return DPD_OK;
 }
@@ -1373,7 +1286,6 @@ void dpd_destroy(dpd_sim *h)
     for (cudaEvent_t e : h->tev) cudaEventDestroy(e);
     if (h->ev) cudaEventDestroy(h->ev);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
-    if (h->side) cudaStreamDestroy(h->side);
     delete h;
 }
 

@@ -2,7 +2,7 @@
 // Gaussian of Sec. 3.5), harmonic bonds (Sec. 4.5), body force (Sec. 4.2),
 // and the velocity-Verlet phases (Sec. 3.1, Algorithm 1): k_force (pairs),
 // k_settle (Newton-3 sums + integration), k_phase1, k_advance (rebuild
-// flag, buffer flip, conditional graph node).
+// flag, buffer flip).
 #include "dpd_internal.cuh"
 #include "dpd_math.cuh"
 
@@ -22,29 +22,16 @@ __device__ __forceinline__ float wrap_pos(float x, float L, float invL)
     return x;
 }
 
-// End of a kernel that moves particles: a block any of whose particles
-// crossed the displacement threshold raises rebuild_next (a plain store of
-// the same value from every such block).  k_advance, launched right after,
-// publishes it and flips the buffer set; no block counts the others.
-__device__ __forceinline__ void finish_block(DevCtl *ctl, bool moved)
-{
-    if (__syncthreads_or(moved) && threadIdx.x == 0) ctl->rebuild_next = 1u;
-}
-
-// One thread, after a moving kernel: the rebuild flag for the chain that
-// follows (also raised when rebuild_every steps have passed), and, when the
-// kernel integrated into the other buffer set, that set becomes the live one
-// and the step advances.  Inside a CUDA graph the flag also sets the
-// conditional node around the next rebuild chain, so a step without a
-// rebuild launches none of the chain's kernels.
+// One thread, once every block of a moving kernel is done: the rebuild flag
+// for the chain that follows (also raised when rebuild_every steps have
+// passed), and, when the kernel integrated into the other buffer set, that set
+// becomes the live one and the step advances.
 template <bool ADVANCE, bool CHECK_EVERY>
-__global__ void k_advance(SimParams P, Ptrs D, NextCond nc)
+__device__ __forceinline__ void advance(const SimParams &P, DevCtl *c)
 {
-    DevCtl *c = D.ctl;
-    uint32_t next = c->rebuild_next;
+    uint32_t next = __ldcg(&c->rebuild_next);
     if (CHECK_EVERY && P.rebuild_every > 0 && c->since_rebuild + 1u >= (uint32_t)P.rebuild_every) next = 1u;
     c->rebuild = next;
-    if (nc.use) cudaGraphSetConditional(nc.handle, next ? 1u : 0u);
     c->rebuild_next = 0u;
     if (ADVANCE) {
         c->parity ^= 1u;
@@ -52,6 +39,38 @@ __global__ void k_advance(SimParams P, Ptrs D, NextCond nc)
         c->since_rebuild += 1u;
     }
 }
+
+template <bool ADVANCE, bool CHECK_EVERY>
+__global__ void k_advance(SimParams P, Ptrs D)
+{
+    dependency_wait();
+    advance<ADVANCE, CHECK_EVERY>(P, D.ctl);
+}
+
+// End of a kernel that moves particles: a block any of whose particles
+// crossed the displacement threshold raises rebuild_next (a plain store of
+// the same value from every such block).  merge: the last block to finish
+// advances; otherwise k_advance does, launched right after.  Every block has
+// read the control words long before it is counted.
+template <bool ADVANCE, bool CHECK_EVERY>
+__device__ __forceinline__ void finish_block(const SimParams &P, DevCtl *ctl, bool moved, int merge)
+{
+    const int any = __syncthreads_or(moved);
+    if (threadIdx.x != 0) return;
+    if (any) ctl->rebuild_next = 1u;
+    if (!merge) return;
+    __threadfence();
+    if (atomicAdd(&ctl->done, 1u) + 1u == gridDim.x) {
+        __threadfence();
+        ctl->done = 0u;
+        advance<ADVANCE, CHECK_EVERY>(P, ctl);
+    }
+}
+
+// Whether the moving kernel's last block advances: up to this many blocks
+// (262,144 particles in Newton-3 mode) counting them costs less than a launch;
+// with 3M particles' 11,700 blocks the atomics on one word cost 33 us a step.
+constexpr int kMergeBlocks = 1024;
 
 __device__ __forceinline__ bool moved_beyond(const SimParams &P, float4 x, float4 r)
 {
@@ -65,8 +84,9 @@ __device__ __forceinline__ bool moved_beyond(const SimParams &P, float4 x, float
 //   u = v + dt/2 f,  x += dt u  (= x + dt v + dt^2/2 f),  v~ = v + lambda dt f
 // (v~ = u when lambda = 1/2), signature for step k+1, displacement check.
 template <bool LHALF>
-__global__ void k_phase1(SimParams P, Ptrs D)
+__global__ void k_phase1(SimParams P, Ptrs D, int merge)
 {
+    dependency_wait();
     DevCtl *ctl = D.ctl;
     const uint32_t par = ctl->parity;
     const uint32_t step1 = (uint32_t)(ctl->step + 1ull);
@@ -96,11 +116,12 @@ __global__ void k_phase1(SimParams P, Ptrs D)
         }
         moved |= moved_beyond(P, x, xr);
     }
-    finish_block(ctl, moved);
+    finish_block<false, true>(P, ctl, moved, merge);
 }
 
 __global__ void k_signature(SimParams P, Ptrs D)
 {
+    dependency_wait();
     const uint32_t par = D.ctl->parity;
     const uint32_t step = (uint32_t)D.ctl->step;
     float4 *vel = D.vel[par];
@@ -447,11 +468,12 @@ __device__ __forceinline__ void block_sum_double(float x, double *out)
 // compiler's 47 registers and 10 blocks; 32 registers spill and take 0.474).
 constexpr int kForceMinBlocks = 12;
 template <bool ONE_SPECIES, int SMODE, int MODE, bool LHALF, bool N3, bool VIR>
-__global__ void __launch_bounds__(kForceThreads, kForceMinBlocks) k_force(SimParams P, Ptrs D, int out_fout)
+__global__ void __launch_bounds__(kForceThreads, kForceMinBlocks) k_force(SimParams P, Ptrs D, int out_fout, int merge)
 {
     constexpr int W = kForceThreads / 32;
     __shared__ WarpSmem s_w[W];
     __shared__ float a_tab[kMaxSpecies * kMaxSpecies];
+    dependency_wait();
     if (!ONE_SPECIES) {
         for (int k = threadIdx.x; k < P.n_species * P.n_species; k += blockDim.x) a_tab[k] = P.a[k];
         __syncthreads();
@@ -511,7 +533,7 @@ __global__ void __launch_bounds__(kForceThreads, kForceMinBlocks) k_force(SimPar
         moved = force_epilogue<MODE, LHALF>(P, D, ctl, i, pi, vi, fx, fy, fz, par, opar, step0, out_fout,
                                             VIR ? &vir : nullptr);
     if (VIR) block_sum_double(vir, D.vir_part + blockIdx.x);
-    if (MODE != kForceEval) finish_block(ctl, moved);
+    if (MODE != kForceEval) finish_block<true, MODE == kForceStep>(P, ctl, moved, merge);
 }
 
 // Row layout (list_layout 1): the paper's force evaluation.  One thread per
@@ -565,9 +587,10 @@ __device__ __forceinline__ void row_pairs(const SimParams &P, const Ptrs &D, con
 }
 
 template <bool ONE_SPECIES, int SMODE, int MODE, bool LHALF, bool VIR>
-__global__ void __launch_bounds__(kForceThreads) k_force_rows(SimParams P, Ptrs D, int out_fout)
+__global__ void __launch_bounds__(kForceThreads) k_force_rows(SimParams P, Ptrs D, int out_fout, int merge)
 {
     __shared__ float a_tab[kMaxSpecies * kMaxSpecies];
+    dependency_wait();
     if (!ONE_SPECIES) {
         for (int k = threadIdx.x; k < P.n_species * P.n_species; k += blockDim.x) a_tab[k] = P.a[k];
         __syncthreads();
@@ -604,7 +627,7 @@ __global__ void __launch_bounds__(kForceThreads) k_force_rows(SimParams P, Ptrs 
         moved = force_epilogue<MODE, LHALF>(P, D, ctl, i, pi, vi, fx, fy, fz, par, opar, step0, out_fout,
                                             VIR ? &vir : nullptr);
     if (VIR) block_sum_double(vir, D.vir_part + blockIdx.x);
-    if (MODE != kForceEval) finish_block(ctl, moved);
+    if (MODE != kForceEval) finish_block<true, MODE == kForceStep>(P, ctl, moved, merge);
 }
 
 // Newton-3 mode: f_i = facc[step & 1][i], the sum of the particle's own-group
@@ -613,8 +636,9 @@ __global__ void __launch_bounds__(kForceThreads) k_force_rows(SimParams P, Ptrs 
 // leaves the buffer to the next step's pair kernel, which clears it; a plain
 // evaluation (the step does not advance) clears it here.
 template <int MODE, bool LHALF>
-__global__ void __launch_bounds__(kThreads) k_settle(SimParams P, Ptrs D, int out_fout)
+__global__ void __launch_bounds__(kThreads) k_settle(SimParams P, Ptrs D, int out_fout, int merge)
 {
+    dependency_wait();
     DevCtl *ctl = D.ctl;
     const uint32_t par = ctl->parity;
     const uint32_t opar = ctl->oparity;
@@ -628,7 +652,7 @@ __global__ void __launch_bounds__(kThreads) k_settle(SimParams P, Ptrs D, int ou
         moved |= integrate_particle<MODE, LHALF>(P, D, ctl, i, pi, vi, f.x, f.y, f.z, par, opar, step0, out_fout);
         if (MODE == kForceEval) facc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    if (MODE != kForceEval) finish_block(ctl, moved);
+    if (MODE != kForceEval) finish_block<true, MODE == kForceStep>(P, ctl, moved, merge);
 }
 
 
@@ -640,71 +664,79 @@ int grid_for(int n)
 
 constexpr int kMaxDynSmem = 160 * 1024;  // largest staging buffer the brick builder accepts
 
-template <bool ONE, int MODE, bool LH, bool N3, bool VIR>
-cudaError_t launch_force_v(const SimParams &P, const Ptrs &D, int of, cudaStream_t s)
+int force_blocks(const SimParams &P)
 {
-    if (!N3 && P.list_layout == 1) {
-        const int gr = (P.n + kForceThreads - 1) / kForceThreads;
-        switch (P.s_mode) {
-        case 1: k_force_rows<ONE, 1, MODE, LH, VIR><<<gr, kForceThreads, 0, s>>>(P, D, of); break;
-        case 2: k_force_rows<ONE, 2, MODE, LH, VIR><<<gr, kForceThreads, 0, s>>>(P, D, of); break;
-        case 3: k_force_rows<ONE, 3, MODE, LH, VIR><<<gr, kForceThreads, 0, s>>>(P, D, of); break;
-        default: k_force_rows<ONE, 0, MODE, LH, VIR><<<gr, kForceThreads, 0, s>>>(P, D, of); break;
+    return P.list_layout == 1 ? (P.n + kForceThreads - 1) / kForceThreads : (P.ngroups + kForceWarps - 1) / kForceWarps;
+}
+
+template <bool ONE, int MODE, bool LH, bool N3, bool VIR>
+cudaError_t launch_force_v(const SimParams &P, const Ptrs &D, int of, cudaStream_t s, bool ov, int merge)
+{
+    const int g = force_blocks(P);
+    if constexpr (!N3) {
+        if (P.list_layout == 1) {
+            switch (P.s_mode) {
+            case 1: return launch_kernel(k_force_rows<ONE, 1, MODE, LH, VIR>, g, kForceThreads, 0, s, ov, P, D, of, merge);
+            case 2: return launch_kernel(k_force_rows<ONE, 2, MODE, LH, VIR>, g, kForceThreads, 0, s, ov, P, D, of, merge);
+            case 3: return launch_kernel(k_force_rows<ONE, 3, MODE, LH, VIR>, g, kForceThreads, 0, s, ov, P, D, of, merge);
+            default: return launch_kernel(k_force_rows<ONE, 0, MODE, LH, VIR>, g, kForceThreads, 0, s, ov, P, D, of, merge);
+            }
         }
-        return cudaGetLastError();
     }
-    const int g = (P.ngroups + kForceWarps - 1) / kForceWarps;
     switch (P.s_mode) {
-    case 1: k_force<ONE, 1, MODE, LH, N3, VIR><<<g, kForceThreads, 0, s>>>(P, D, of); break;
-    case 2: k_force<ONE, 2, MODE, LH, N3, VIR><<<g, kForceThreads, 0, s>>>(P, D, of); break;
-    case 3: k_force<ONE, 3, MODE, LH, N3, VIR><<<g, kForceThreads, 0, s>>>(P, D, of); break;
-    default: k_force<ONE, 0, MODE, LH, N3, VIR><<<g, kForceThreads, 0, s>>>(P, D, of); break;
+    case 1: return launch_kernel(k_force<ONE, 1, MODE, LH, N3, VIR>, g, kForceThreads, 0, s, ov, P, D, of, merge);
+    case 2: return launch_kernel(k_force<ONE, 2, MODE, LH, N3, VIR>, g, kForceThreads, 0, s, ov, P, D, of, merge);
+    case 3: return launch_kernel(k_force<ONE, 3, MODE, LH, N3, VIR>, g, kForceThreads, 0, s, ov, P, D, of, merge);
+    default: return launch_kernel(k_force<ONE, 0, MODE, LH, N3, VIR>, g, kForceThreads, 0, s, ov, P, D, of, merge);
     }
-    return cudaGetLastError();
 }
 
 // The virial is taken by every evaluation except the inner steps of a run.
 template <bool ONE, int MODE, bool LH, bool N3>
-cudaError_t launch_force_m(const SimParams &P, const Ptrs &D, int of, cudaStream_t s, bool vir)
+cudaError_t launch_force_m(const SimParams &P, const Ptrs &D, int of, cudaStream_t s, bool vir, bool ov, int merge)
 {
-    return vir ? launch_force_v<ONE, MODE, LH, N3, true>(P, D, of, s) : launch_force_v<ONE, MODE, LH, N3, false>(P, D, of, s);
+    return vir ? launch_force_v<ONE, MODE, LH, N3, true>(P, D, of, s, ov, merge)
+               : launch_force_v<ONE, MODE, LH, N3, false>(P, D, of, s, ov, merge);
 }
 
+// one thread per particle: the settle kernel streams memory and needs every
+// load in flight at once
+int settle_blocks(const SimParams &P) { return (P.n + kThreads - 1) / kThreads; }
+
+bool merged(const SimParams &P) { return (P.newton3 ? settle_blocks(P) : force_blocks(P)) <= kMergeBlocks; }
+
 template <bool ONE>
-cudaError_t launch_force_s(const SimParams &P, const Ptrs &D, int mode, int of, cudaStream_t s, cudaEvent_t after_pair,
-                           unsigned int ev_flags, NextCond nc)
+cudaError_t launch_force_s(const SimParams &P, const Ptrs &D, int mode, int of, cudaStream_t s, bool ov,
+                           cudaEvent_t after_pair, unsigned int ev_flags)
 {
+    const int merge = merged(P) ? 1 : 0;
+    cudaError_t e;
     if (P.newton3) {
         // pair kernel (accumulation only), then the settle kernel of the mode
-        cudaError_t e = launch_force_m<ONE, kForceEval, true, true>(P, D, of, s, mode != kForceStep);
+        e = launch_force_m<ONE, kForceEval, true, true>(P, D, of, s, mode != kForceStep, ov, merge);
         if (e == cudaSuccess && after_pair) e = cudaEventRecordWithFlags(after_pair, s, ev_flags);
         if (e != cudaSuccess) return e;
-        // one thread per particle: the kernel streams memory and needs every
-        // load in flight at once
-        const int g = (P.n + kThreads - 1) / kThreads;
-        if (mode == kForceEval) k_settle<kForceEval, true><<<g, kThreads, 0, s>>>(P, D, of);
-        else if (P.lambda_half) {
-            if (mode == kForceStep) k_settle<kForceStep, true><<<g, kThreads, 0, s>>>(P, D, of);
-            else k_settle<kForceFinish, true><<<g, kThreads, 0, s>>>(P, D, of);
-        } else {
-            if (mode == kForceStep) k_settle<kForceStep, false><<<g, kThreads, 0, s>>>(P, D, of);
-            else k_settle<kForceFinish, false><<<g, kThreads, 0, s>>>(P, D, of);
-        }
-    } else {
-        cudaError_t e;
-        if (mode == kForceEval) e = launch_force_m<ONE, kForceEval, true, false>(P, D, of, s, true);
+        const int gs = settle_blocks(P);
+        if (mode == kForceEval) e = launch_kernel(k_settle<kForceEval, true>, gs, kThreads, 0, s, ov, P, D, of, merge);
         else if (P.lambda_half)
-            e = mode == kForceStep ? launch_force_m<ONE, kForceStep, true, false>(P, D, of, s, false)
-                                   : launch_force_m<ONE, kForceFinish, true, false>(P, D, of, s, true);
+            e = mode == kForceStep ? launch_kernel(k_settle<kForceStep, true>, gs, kThreads, 0, s, ov, P, D, of, merge)
+                                   : launch_kernel(k_settle<kForceFinish, true>, gs, kThreads, 0, s, ov, P, D, of, merge);
         else
-            e = mode == kForceStep ? launch_force_m<ONE, kForceStep, false, false>(P, D, of, s, false)
-                                   : launch_force_m<ONE, kForceFinish, false, false>(P, D, of, s, true);
+            e = mode == kForceStep ? launch_kernel(k_settle<kForceStep, false>, gs, kThreads, 0, s, ov, P, D, of, merge)
+                                   : launch_kernel(k_settle<kForceFinish, false>, gs, kThreads, 0, s, ov, P, D, of, merge);
+    } else {
+        if (mode == kForceEval) e = launch_force_m<ONE, kForceEval, true, false>(P, D, of, s, true, ov, merge);
+        else if (P.lambda_half)
+            e = mode == kForceStep ? launch_force_m<ONE, kForceStep, true, false>(P, D, of, s, false, ov, merge)
+                                   : launch_force_m<ONE, kForceFinish, true, false>(P, D, of, s, true, ov, merge);
+        else
+            e = mode == kForceStep ? launch_force_m<ONE, kForceStep, false, false>(P, D, of, s, false, ov, merge)
+                                   : launch_force_m<ONE, kForceFinish, false, false>(P, D, of, s, true, ov, merge);
         if (e == cudaSuccess && after_pair) e = cudaEventRecordWithFlags(after_pair, s, ev_flags);
-        if (e != cudaSuccess) return e;
     }
-    if (mode == kForceStep) k_advance<true, true><<<1, 1, 0, s>>>(P, D, nc);
-    else if (mode == kForceFinish) k_advance<true, false><<<1, 1, 0, s>>>(P, D, nc);
-    return cudaGetLastError();
+    if (e != cudaSuccess || merge || mode == kForceEval) return e;
+    return mode == kForceStep ? launch_kernel(k_advance<true, true>, 1, 1, 0, s, ov, P, D)
+                              : launch_kernel(k_advance<true, false>, 1, 1, 0, s, ov, P, D);
 }
 
 }  // namespace
@@ -721,22 +753,24 @@ cudaError_t launch_signature(const SimParams &P, const Ptrs &D, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_phase1(const SimParams &P, const Ptrs &D, cudaStream_t s, NextCond nc)
+cudaError_t launch_phase1(const SimParams &P, const Ptrs &D, cudaStream_t s, bool overlap)
 {
-    const int g = (P.n + kThreads - 1) / kThreads;
-    if (P.lambda_half)
-        k_phase1<true><<<g, kThreads, 0, s>>>(P, D);
-    else
-        k_phase1<false><<<g, kThreads, 0, s>>>(P, D);
-    k_advance<false, true><<<1, 1, 0, s>>>(P, D, nc);
-    return cudaGetLastError();
+    const int g = settle_blocks(P), merge = g <= kMergeBlocks ? 1 : 0;
+    cudaError_t e = P.lambda_half ? launch_kernel(k_phase1<true>, g, kThreads, 0, s, overlap, P, D, merge)
+                                  : launch_kernel(k_phase1<false>, g, kThreads, 0, s, overlap, P, D, merge);
+    if (e != cudaSuccess || merge) return e;
+    return launch_kernel(k_advance<false, true>, 1, 1, 0, s, overlap, P, D);
 }
 
-cudaError_t launch_force(const SimParams &P, const Ptrs &D, int mode, bool out_fout, cudaStream_t s,
-                         cudaEvent_t after_pair, unsigned int ev_flags, NextCond nc)
+int phase1_kernels(const SimParams &P) { return settle_blocks(P) <= kMergeBlocks ? 1 : 2; }
+
+int force_kernels(const SimParams &P) { return 1 + (P.newton3 ? 1 : 0) + (merged(P) ? 0 : 1); }
+
+cudaError_t launch_force(const SimParams &P, const Ptrs &D, int mode, bool out_fout, cudaStream_t s, bool overlap,
+                         cudaEvent_t after_pair, unsigned int ev_flags)
 {
-    if (P.n_species == 1) return launch_force_s<true>(P, D, mode, out_fout ? 1 : 0, s, after_pair, ev_flags, nc);
-    return launch_force_s<false>(P, D, mode, out_fout ? 1 : 0, s, after_pair, ev_flags, nc);
+    if (P.n_species == 1) return launch_force_s<true>(P, D, mode, out_fout ? 1 : 0, s, overlap, after_pair, ev_flags);
+    return launch_force_s<false>(P, D, mode, out_fout ? 1 : 0, s, overlap, after_pair, ev_flags);
 }
 
 }  // namespace dpd

@@ -221,6 +221,9 @@ cudaError_t launch_import(const SimParams &P, const double box[3], int64_t n, co
                           const int32_t *sp, const uint32_t *tag, float4 *pos, float4 *vel, uint32_t *tag_out,
                           uint32_t *pid_out, cudaStream_t s);
 cudaError_t launch_export(int64_t n, const float4 *src, const uint32_t *pid, double *out, cudaStream_t s);
+// profile: nblocks = profile_blocks_for(n, nbins) partials of 2 nbins in D.red,
+// then their fixed-order sum (sum, count by bin) behind them
+int profile_blocks_for(int64_t n, int nbins);
 cudaError_t launch_profile(const SimParams &P, const Ptrs &D, int bin_axis, int vel_axis, int nbins,
                            int nblocks, cudaStream_t s);
 cudaError_t launch_pair_rng(uint64_t seed, uint64_t step, int64_t m, const uint32_t *ti, const uint32_t *tj,

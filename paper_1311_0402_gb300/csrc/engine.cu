@@ -1170,8 +1170,8 @@ dpd_status dpd_profile(dpd_sim *h, int32_t bin_axis, int32_t vel_axis, int32_t n
     if (bin_axis < 0 || bin_axis > 2 || vel_axis < 0 || vel_axis > 2 || nbins < 1 || nbins > 100000 || !sum_out ||
         !count_out)
         return fail(h, DPD_ERR_ARG, "invalid profile arguments");
-    int nblocks = (int)std::min<int64_t>(std::max<int64_t>(1, h->n / 1024), 1024);
-    size_t need = (size_t)nblocks * 2 * nbins;
+    const int nblocks = profile_blocks_for(h->n, nbins);
+    const size_t parts = (size_t)nblocks * 2 * nbins, need = parts + 2 * (size_t)nbins;
     if (need > h->red_doubles) {
         double *nr = nullptr;
         st = dev_alloc(h, (void **)&nr, need * sizeof(double), h->allocs);
@@ -1182,15 +1182,14 @@ dpd_status dpd_profile(dpd_sim *h, int32_t bin_axis, int32_t vel_axis, int32_t n
         drop_graphs(h);
     }
     CUDA_TRY(h, launch_profile(h->P, h->D, bin_axis, vel_axis, nbins, nblocks, h->stream));
-    std::vector<double> part(need);
-    CUDA_TRY(h, cudaMemcpyAsync(part.data(), h->D.red, sizeof(double) * need, cudaMemcpyDeviceToHost, h->stream));
+    std::vector<double> sums(2 * (size_t)nbins);
+    CUDA_TRY(h, cudaMemcpyAsync(sums.data(), h->D.red + parts, sizeof(double) * sums.size(), cudaMemcpyDeviceToHost, h->stream));
     st = wait(h);
     if (st) return st;
-    for (int b = 0; b < nblocks; ++b)
-        for (int k = 0; k < nbins; ++k) {
-            sum_out[k] += part[((size_t)b * nbins + k) * 2];
-            count_out[k] += part[((size_t)b * nbins + k) * 2 + 1];
-        }
+    for (int k = 0; k < nbins; ++k) {
+        sum_out[k] += sums[2 * (size_t)k];
+        count_out[k] += sums[2 * (size_t)k + 1];
+    }
     return DPD_OK;
 }
 

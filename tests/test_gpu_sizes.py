@@ -63,3 +63,59 @@ def test_fixed_capacity_keeps_the_shared_capacity_of_32():
         return out
     a, b = forces(0), forces(24)
     assert force_error(a, b)[0] < FORCE_TOL
+
+
+# the one-launch sort up to 4,096 particles and cells; 8 lanes a particle up to
+# 20,000, 4 up to 50,000, else 2; one, two and more cells along an axis; more
+# pairs than a lane notes (rho = 24)
+@pytest.mark.parametrize("n,box,s", [(1, (3.0, 4.0, 5.0), 1.0), (40, (2.1, 2.1, 2.1), 1.0), (98, (2.05, 3.1, 6.0), 0.5),
+                                     (700, (4.5, 4.5, 4.5), 0.25), (3000, (5.0, 5.0, 5.0), 1.0),
+                                     (4096, (11.0, 12.0, 10.0), 1.0), (4097, (11.0, 12.0, 10.0), 2.0),
+                                     (1000, (17.0, 16.0, 16.0), 1.0), (20000, (20.0, 18.0, 19.0), 0.5),
+                                     (20001, (20.0, 18.0, 19.0), 1.0), (50001, (26.0, 25.0, 25.5), 1.0),
+                                     (131072, (35.2, 36.0, 34.3), 0.5), (60000, (40.0, 41.0, 39.9), 1.0)])
+def test_static_forces_each_side_of_the_size_rules(n, box, s):
+    need_gpu()
+    import torch
+    x, v = workloads.uniform_fluid(box, n, 1.0, n + 1)[:2]
+    x32 = np.minimum(x.astype(np.float32), np.nextafter(np.asarray(box, np.float32), np.float32(0.0)))
+    v32 = v.astype(np.float32)
+    sp = np.random.default_rng(n).integers(0, 2, n).astype(np.int32)
+    a = [[25.0, 40.0], [40.0, 30.0]]
+    prm = dpd.dpd_static_params_from(box, a, 4.5, 1.0, 1.0, s, 0.01, seed=9, body_mode=2, body=(0.3, 0.0, -0.1))
+    pos, vel = torch.zeros((n, 4)), torch.zeros((n, 4))
+    pos[:, :3], vel[:, :3] = torch.from_numpy(x32), torch.from_numpy(v32)
+    pos[:, 3] = torch.from_numpy(sp.view(np.float32))
+    pos, vel, out = pos.cuda(), vel.cuda(), torch.full((n, 4), float("nan"), device="cuda")
+    got = []
+    for _ in range(2):
+        dpd.dpd_forces_static(prm, n, pos.data_ptr(), vel.data_ptr(), None, 4, out.data_ptr(),
+                              torch.cuda.current_stream().cuda_stream)
+        got.append(out.cpu().numpy().copy())
+    assert np.array_equal(got[0], got[1])  # fixed order: the same bits
+    o = oracle.System(box, a, 4.5, 1.0, 1.0, s, 0.01, seed=9, body_mode=2, body=(0.3, 0.0, -0.1), cut_fp32=True)
+    f, _ = o.forces(x32.astype(np.float64), v32.astype(np.float64), species=sp, step=4)
+    assert force_error(got[0][:, :3].astype(np.float64), f)[0] < FORCE_TOL
+
+
+# a table per warp up to 512 bins, fewer warps up to 4,096, each bin its own
+# scan above; FP64 sums of FP32 values: 1e-12 of the largest sum is far above
+# their rounding (n 2^-53)
+@pytest.mark.parametrize("n,nbins", [(1, 1), (500, 3), (3000, 60), (30000, 512), (30000, 513), (9000, 4096), (9000, 4097)])
+def test_profile_each_side_of_the_size_rules(n, nbins):
+    need_gpu()
+    c = workloads.CONFIGS["fluid_small"]
+    box = (10.0, 11.0, 12.0)
+    x, v = workloads.uniform_fluid(box, n, 1.0, n)[:2]
+    g = dpd.Sim(box, c["a"], c["gamma"], c["kT"], c["rc"], c["s"], c["dt"])
+    g.set_state(x, v)
+    x32, v32, _ = g.state()
+    for axis, comp in ((1, 0), (2, 2)):
+        b = (x32[:, axis].astype(np.float32) * (np.float32(nbins) / np.float32(box[axis]))).astype(np.int64)
+        b = np.clip(b, 0, nbins - 1)
+        start = np.arange(nbins, dtype=np.float64)
+        sums, counts = g.profile(axis, comp, nbins, start.copy(), start.copy())
+        ref = np.bincount(b, weights=v32[:, comp], minlength=nbins)
+        assert np.array_equal(counts - start, np.bincount(b, minlength=nbins))
+        assert np.abs(sums - start - ref).max() < 1e-12 * max(np.abs(ref).max(), nbins, 1.0)
+    g.close()

@@ -26,7 +26,13 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+struct dpd_sim;
+
 namespace dpd {
+
+// How many handles are expected to run side by side on the device (before the
+// first dpd_set_state; 1 unless called): each is then launched for its share.
+void expect_concurrent(dpd_sim *h, int handles);
 
 constexpr int kMaxSpecies = 8;
 constexpr int kMaxBonds = 6;          // bonds per particle

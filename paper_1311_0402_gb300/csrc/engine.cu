@@ -148,6 +148,7 @@ struct dpd_sim {
     std::string err;
     std::vector<uint32_t> bond_partner_host;
     bool bonds_set = false;
+    int share = 1;                           // handles expected to run side by side (expect_concurrent)
 };
 
 namespace {
@@ -340,17 +341,23 @@ cudaError_t enqueue_steps_timed(dpd_sim *h, int64_t k)
     return e;
 }
 
+// Whether a handle's kernels overlap their launches.  Of three handles side by
+// side and more, the kernels that wait early take the room the others' work
+// would fill.
+bool overlaps(const dpd_sim *h) { return h->share < 3; }
+
 // Kernel sequence of k steps (starting and ending at a full-step state):
 // phase 1, then per step the rebuild chain (its kernels return at once unless
 // flagged), the pair kernel and the integration into the next step (or the
 // finish of the last).
 cudaError_t enqueue_steps(dpd_sim *h, int64_t k)
 {
-    cudaError_t e = launch_phase1(h->P, h->D, h->stream, true);
+    const bool ov = overlaps(h);
+    cudaError_t e = launch_phase1(h->P, h->D, h->stream, ov);
     for (int64_t s = 0; s < k && e == cudaSuccess; ++s) {
-        e = launch_rebuild(h->P, h->D, h->stream, h->n_scan_blocks, true);
+        e = launch_rebuild(h->P, h->D, h->stream, h->n_scan_blocks, ov);
         if (e == cudaSuccess)
-            e = launch_force(h->P, h->D, s + 1 < k ? kForceStep : kForceFinish, false, h->stream, true);
+            e = launch_force(h->P, h->D, s + 1 < k ? kForceStep : kForceFinish, false, h->stream, ov);
     }
     return e;
 }
@@ -410,6 +417,9 @@ int group_count(const dpd_sim *h, int64_t n)
 // 33.5; 81,000 56.7 / 44.6 / 43.2 / 45.7; 207,000 73.5 / 68.4 / 69.6 / -;
 // 648,000 155.3 / 156.0 / - / -; 3,000,000 575 / 604 / - / -, and a split of
 // 2 there 591.  A fixed capacity keeps groups of 32, whose particles share it.
+// Handles that run side by side each want their share of the chip only (in
+// deterministic mode the groups, which order the sums, stay those of a handle
+// alone).
 void pick_groups(dpd_sim *h, int64_t n)
 {
     SimParams &P = h->P;
@@ -417,9 +427,9 @@ void pick_groups(dpd_sim *h, int64_t n)
     P.brick_split = 1;
     if (!P.use_bricks) return;
     if (P.list_layout == 0 && h->opt.nbr_capacity == 0)
-        while (P.group > kMinGroup && n < (int64_t)kGroupsWanted * P.group) P.group /= 2;
+        while (P.group > kMinGroup && n < (int64_t)(kGroupsWanted / (h->P.newton3 ? h->share : 1)) * P.group) P.group /= 2;
     const int64_t rounds = (n / P.nbricks + P.group * kBuildWarps - 1) / (P.group * kBuildWarps);
-    P.brick_split = (int)std::max<int64_t>(1, std::min<int64_t>(kBuildBlocksWanted / P.nbricks, rounds));
+    P.brick_split = (int)std::max<int64_t>(1, std::min<int64_t>(kBuildBlocksWanted / h->share / P.nbricks, rounds));
 }
 
 // per-particle capacity from the largest group total of a build
@@ -540,6 +550,16 @@ dpd_status download_xyz(dpd_sim *h, const float4 *dev, double *out)
 }
 
 }  // namespace
+
+namespace dpd {
+
+// At most 8: with 24 boxes of L = 6..30 (1,000 steps each, all at once) the
+// serving loop took 248 ms with every handle launched as if alone, 196 at a
+// share of 3, 180 at 8 and 176 at 24, where few boxes at a time run slower
+// (two of L = 20: 36, 35, 40 and 52 ms).
+void expect_concurrent(dpd_sim *h, int handles) { h->share = std::min(std::max(handles, 1), 8); }
+
+}  // namespace dpd
 
 extern "C" {
 

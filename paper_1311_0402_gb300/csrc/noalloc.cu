@@ -407,7 +407,8 @@ template <int SMODE, int T>
 __global__ void __launch_bounds__(kNAForceThreads) k_na_force(NAParams P, NAScratch S, float4 *fout)
 {
     __shared__ NAWarp<T> s_warp[kNAForceThreads / 32];
-    dependency_wait();
+    // (no launch_dependents: what the caller launches next starts afterwards)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t p = (uint32_t)(t / T);
     const int sub = t % T;

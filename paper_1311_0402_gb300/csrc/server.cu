@@ -182,6 +182,11 @@ dpd_status start(dpd_server *S, Slot &sl)
     o.stream = nullptr;  // a stream of the box's own
     dpd_status st = dpd_create(&sl.sim, sl.job.box, sl.job.n_species, sl.job.a.data(), sl.job.gamma, sl.job.kT,
                                sl.job.rc, sl.job.s, sl.job.dt, &o);
+    if (st == DPD_OK) {
+        std::lock_guard<std::mutex> lk(S->m);
+        const int64_t waiting = S->handle_active + (int64_t)S->pending.size();
+        dpd::expect_concurrent(sl.sim, (int)std::min<int64_t>(waiting, S->opt.max_active));
+    }
     if (st != DPD_OK) {
         sl.sim = nullptr;
         return st;

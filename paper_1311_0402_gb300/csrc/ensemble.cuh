@@ -14,7 +14,13 @@ namespace dpd {
 constexpr int kEnsQueue = 64;      // hit ring per warp (< 32 pending + 32 new)
 constexpr int kEnsSlots = 4;       // candidates per lane per round, held in registers
 constexpr int kEnsCand = 32 * kEnsSlots;  // candidate buffer per warp (a cell's 27-cell stencil, in rounds)
-constexpr int kEnsUnitCells = 8;   // consecutive cells per work unit (one warp, queue flushed at the end)
+constexpr int kEnsUnitCells = 8;   // Newton-3 mode: consecutive cells per work unit (one warp, queue flushed at the end)
+constexpr int kEnsLanes = 2;       // default mode: lanes that share a particle
+constexpr int kEnsRanges = 2 * ((9 + kEnsLanes - 1) / kEnsLanes);  // index ranges a lane walks, at most
+constexpr int kEnsNotes = 16;      // pairs a lane notes before they are evaluated
+// per-warp scratch: ranges and notes, or (Newton-3 mode) ring and candidates
+constexpr int kEnsWarpBytes = 32 * (4 * kEnsRanges + 2 * kEnsNotes);
+static_assert(kEnsWarpBytes >= 16 * kEnsQueue + 4 * kEnsCand, "the ring and the candidates share the scratch");
 constexpr int kEnsMaxCluster = 8;  // portable cluster size
 constexpr int kEnsMaxN = 65535;    // particle indices are 16-bit
 
@@ -42,11 +48,10 @@ __host__ __device__ inline size_t ens_align16(size_t b) { return (b + 15) & ~siz
 
 // Dynamic shared memory of one CTA, in this order: pos, u (the velocity the
 // pair force reads, + signature), vh (lambda != 1/2 only), f, cell starts
-// [ncell + 1], cell counts [ncell], sorted indices [n], arrival slots [n],
-// owning CTA of each particle this step [n] (Newton-3 mode), then per warp
-// the hit ring and the candidate buffer.
+// [ncell + 1], cell counts [ncell], sorted indices [n], owning CTA of each
+// particle this step [n] (Newton-3 mode), then the warps' scratch.
 struct EnsLayout {
-    size_t pos, u, vh, f, start, cnt, idx, slot, own, q, cand, total;
+    size_t pos, u, vh, f, start, cnt, idx, own, warp, total;
 };
 
 __host__ __device__ inline EnsLayout ens_layout(int n, int ncell, bool lhalf, int threads)
@@ -60,11 +65,8 @@ __host__ __device__ inline EnsLayout ens_layout(int n, int ncell, bool lhalf, in
     l.start = o; o += ens_align16((size_t)(ncell + 1) * 4);
     l.cnt = o; o += ens_align16((size_t)ncell * 4);
     l.idx = o; o += ens_align16((size_t)n * 2);
-    l.slot = o; o += ens_align16((size_t)n * 2);
     l.own = o; o += ens_align16((size_t)n);
-    const int warps = threads / 32;
-    l.q = o; o += (size_t)warps * kEnsQueue * 16;
-    l.cand = o; o += (size_t)warps * kEnsCand * 4;
+    l.warp = o; o += (size_t)(threads / 32) * kEnsWarpBytes;
     l.total = o;
     return l;
 }

@@ -8,37 +8,38 @@
 //   1. bins the box into cells of side >= r_c (the cell list of Sec. 3.2.3):
 //      a counting sort by shared-memory atomics, then each cell's members put
 //      in index order, so every replica holds the same cell lists;
-//   2. evaluates the pair forces of its share of the cells: work units of
-//      consecutive cells go round-robin to the cluster's CTAs and their warps.
-//      A warp takes a unit cell by cell; a cell's 27-cell stencil (Sec.
-//      3.3.1) is gathered in rounds of 128 candidates, each lane holding 4 in
-//      registers, and every owner of the cell tests them 32 at a time.  Lane
-//      l < 27 keeps neighbour cell l's periodic shift s; a slot holding a
-//      shifted candidate fetches it by shuffle and forms (x_j - x_i) + s, the
-//      rounding of the other kernels' FP32 predicate.  Hits inside r_c go to
-//      a per-warp ring in shared memory, evaluated 32 pairs at a time by the
-//      whole warp (Eqs. 2-9, the TEA hash and Box-Muller Gaussian of Sec.
-//      3.5), and summed per owner by a segmented shuffle scan (each pair is
-//      seen from both sides).
-//      Within a candidate round every owner's hits are one run of the ring;
-//      the ring is emptied between rounds, so a batch never holds two runs of
-//      one owner.  In the optional Newton-3 mode the stencil is halved (the
-//      own cell's later members and the 13 forward cells) and the partner's
-//      share goes by an atomic to the shared memory of the CTA that
-//      integrates it;
-//   3. integrates the particles of its cells (the lambda form of velocity
-//      Verlet, Sec. 3.1 / Algorithm 1) and stores their new state into every
-//      replica of the cluster through distributed shared memory.
+//   2. evaluates the pair forces of its share of the particles: runs of
+//      consecutive particles in cell order go round-robin to the cluster's CTAs
+//      and their warps, kEnsLanes lanes a particle.  A particle's 27-cell stencil
+//      (Sec. 3.3.1) is nine rows of cells, each one or two index ranges of the
+//      sorted particles, dealt to its lanes in turn.  A lane tests the candidates
+//      of its ranges, kEnsBurst loads in flight, as (x_j - x_i) + s with the
+//      range's periodic shift s, the rounding of the other kernels' FP32
+//      predicate, and notes those inside r_c in shared memory; when a lane's
+//      notes run out the warp evaluates them together, each lane its own (Eqs.
+//      2-9, the TEA hash and Box-Muller Gaussian of Sec. 3.5), and the lanes'
+//      sums are added by shuffles (each pair is seen from both sides).  One
+//      candidate in six is a pair, so evaluating a pair as it is met would leave
+//      most lanes idle most of the time.
+//      In the optional Newton-3 mode the stencil is halved (the own cell's later
+//      members and the 13 forward cells): work units of consecutive cells, whose
+//      candidates a warp holds in registers for every owner of the cell and
+//      whose pairs it evaluates 32 at a time from a ring in shared memory, sum
+//      per owner by a segmented shuffle scan, and the partner's share goes by an
+//      atomic to the shared memory of the CTA that integrates it;
+//   3. integrates its particles (the lambda form of velocity Verlet, Sec. 3.1 /
+//      Algorithm 1) and stores their new state into every replica of the cluster
+//      through distributed shared memory.
 // Two cluster barriers per step separate the reads of a step from the
 // writes of the next (a third, in Newton-3 mode with more than one CTA per
 // box, orders the zeroing of every replica's accumulators before any remote
 // add).  The last step writes positions, full-step velocities and forces
 // (w = the particle's virial share) to device memory.
 //
-// Fixed summation order (the default mode): units never span a queue flush, a
-// cell's members are in index order and the stencil order is fixed, so a force
-// does not depend on the cluster size, the block size or the other boxes of
-// the launch.
+// Fixed summation order (the default mode): a particle's lanes walk its ranges
+// in a fixed order, a cell's members are in index order and kEnsLanes is a
+// constant, so a force does not depend on the cluster size, the block size or
+// the other boxes of the launch.
 #include "dpd_math.cuh"
 #include "ensemble.cuh"
 
@@ -80,13 +81,14 @@ __device__ __forceinline__ int ens_cell(const EnsBox &B, float4 p)
 struct EnsPtrs {
     float4 *pos, *u, *vh, *f;
     uint32_t *start, *cnt;
-    uint16_t *idx, *slot;
+    uint16_t *idx;
     uint8_t *own;  // Newton-3 mode: the cluster rank that integrates each particle this step
     int C, rank;   // CTAs per box, this CTA's rank
 };
 
-// Exclusive scan of cnt[0, ncell) into start[0, ncell], start[ncell] = total.
-__device__ void ens_scan(const uint32_t *cnt, uint32_t *start, int ncell, uint32_t *wsum)
+// Exclusive scan of cnt[0, ncell) into start[0, ncell], start[ncell] = total;
+// cnt becomes a copy of the starts.
+__device__ void ens_scan(uint32_t *cnt, uint32_t *start, int ncell, uint32_t *wsum)
 {
     const int T = blockDim.x, t = threadIdx.x, lane = t & 31, warp = t >> 5, nw = T >> 5;
     const int per = (ncell + T - 1) / T;
@@ -115,8 +117,10 @@ __device__ void ens_scan(const uint32_t *cnt, uint32_t *start, int ncell, uint32
     __syncthreads();
     uint32_t run = wsum[warp] + incl - sum;
     for (int c = lo; c < hi; ++c) {
+        const uint32_t k = cnt[c];
         start[c] = run;
-        run += cnt[c];
+        cnt[c] = run;
+        run += k;
     }
     if (t == 0) start[ncell] = wsum[32];
     __syncthreads();
@@ -124,7 +128,7 @@ __device__ void ens_scan(const uint32_t *cnt, uint32_t *start, int ncell, uint32
 
 // Evaluate ring entries [head, head + nb) (nb <= 32), one pair per lane, and
 // add the sums of each run of equal owners to the owner's accumulator.
-template <int SMODE, bool VIR, bool N3>
+template <int SMODE, bool VIR>
 __device__ __forceinline__ void ens_batch(const EnsBox &B, const EnsPtrs &S, const float4 *q, const uint32_t (&key)[4],
                                           uint32_t head, int nb, int lane)
 {
@@ -158,18 +162,17 @@ __device__ __forceinline__ void ens_batch(const EnsBox &B, const EnsPtrs &S, con
         float a = B.a[0];
         if (B.n_species > 1) a = B.a[__float_as_int(S.pos[i].w) * B.n_species + __float_as_int(S.pos[j].w)];
         const float F = fmaf(a, wgt, fmaf(-B.gamma * wR * wR, ev, B.sigma_isdt * wR * xi));
-        if (VIR) fw = N3 ? a * wgt * r : 0.5f * (a * wgt * r);  // once per pair, or from both ends
+        if (VIR) fw = a * wgt * r;  // once per pair
         const float sc = -F * inv_r;
         fx = sc * dx;
         fy = sc * dy;
         fz = sc * dz;
-        if (N3) {  // Newton's third law: the partner gets -F e_ij, in its owner's shared memory
-            float4 *fj = S.f;
-            if (S.C > 1 && (int)S.own[j] != S.rank) fj = cg::this_cluster().map_shared_rank(S.f, (int)S.own[j]);
-            atomicAdd(&fj[j].x, -fx);
-            atomicAdd(&fj[j].y, -fy);
-            atomicAdd(&fj[j].z, -fz);
-        }
+        // Newton's third law: the partner gets -F e_ij, in its owner's shared memory
+        float4 *fj = S.f;
+        if (S.C > 1 && (int)S.own[j] != S.rank) fj = cg::this_cluster().map_shared_rank(S.f, (int)S.own[j]);
+        atomicAdd(&fj[j].x, -fx);
+        atomicAdd(&fj[j].y, -fy);
+        atomicAdd(&fj[j].z, -fz);
     }
     // segmented inclusive scan over runs of equal owners (fixed order)
     const uint32_t prev = __shfl_up_sync(0xFFFFFFFFu, owner, 1);
@@ -191,27 +194,19 @@ __device__ __forceinline__ void ens_batch(const EnsBox &B, const EnsPtrs &S, con
     }
     const uint32_t next = __shfl_down_sync(0xFFFFFFFFu, owner, 1);
     if (lane < nb && (lane == 31 || next != owner)) {
-        if (N3) {  // other warps add partner shares to the same accumulator
-            atomicAdd(&S.f[owner].x, fx);
-            atomicAdd(&S.f[owner].y, fy);
-            atomicAdd(&S.f[owner].z, fz);
-            if (VIR) atomicAdd(&S.f[owner].w, fw);
-        } else {
-            float4 acc = S.f[owner];
-            acc.x += fx;
-            acc.y += fy;
-            acc.z += fz;
-            if (VIR) acc.w += fw;
-            S.f[owner] = acc;
-        }
+        // other warps add partner shares to the same accumulator
+        atomicAdd(&S.f[owner].x, fx);
+        atomicAdd(&S.f[owner].y, fy);
+        atomicAdd(&S.f[owner].z, fz);
+        if (VIR) atomicAdd(&S.f[owner].w, fw);
     }
     __syncwarp();
 }
 
-// Pair forces of the owners in work unit u (cells [u K, u K + K)) into S.f.
-// N3: half stencil (the own cell's later members and the 13 forward cells),
-// the partner's share added by a shared-memory atomic.
-template <int SMODE, bool VIR, bool N3>
+// Newton-3 mode: pair forces of the owners in work unit u (cells [u K, u K + K))
+// into S.f over the half stencil (the own cell's later members and the 13
+// forward cells), the partner's share added by a shared-memory atomic.
+template <int SMODE, bool VIR>
 __device__ void ens_unit(const EnsBox &B, const EnsPtrs &S, float4 *q, uint32_t *cand, int u, int lane)
 {
     const uint32_t key[4] = {B.key[0], B.key[1], B.key[2], B.key[3]};
@@ -222,21 +217,16 @@ __device__ void ens_unit(const EnsBox &B, const EnsPtrs &S, float4 *q, uint32_t 
     for (int c = c0; c < c1; ++c) {
         const int ob = (int)S.start[c], oe = (int)S.start[c + 1];
         if (ob == oe) continue;
-        if (!N3)
-            for (int k = ob + lane; k < oe; k += 32) S.f[S.idx[k]] = make_float4(0.f, 0.f, 0.f, 0.f);
-        // lane l < 27: neighbour cell l of the stencil, its member range and shift
+        // lane 0: the own cell; lanes 1..13: the forward offsets; their member ranges and shifts
         const int cx = c % ncx, cy = (c / ncx) % ncy, cz = c / (ncx * ncy);
         // (the shift stays in the lane's registers; a candidate fetches it by shuffle)
         int len = 0, sbeg = 0;
         float shx = 0.f, shy = 0.f, shz = 0.f;
-        if (lane < (N3 ? 14 : 27)) {
-            int ox = lane % 3 - 1, oy = (lane / 3) % 3 - 1, oz = lane / 9 - 1;
-            if (N3) {  // lane 0: the own cell; lanes 1..13: the forward offsets
-                const int k = lane - 1;
-                ox = lane == 0 ? 0 : (k < 9 ? k % 3 - 1 : (k < 12 ? k - 10 : 1));
-                oy = lane == 0 ? 0 : (k < 9 ? k / 3 - 1 : (k < 12 ? 1 : 0));
-                oz = lane == 0 ? 0 : (k < 9 ? 1 : 0);
-            }
+        if (lane < 14) {
+            const int k = lane - 1;
+            const int ox = lane == 0 ? 0 : (k < 9 ? k % 3 - 1 : (k < 12 ? k - 10 : 1));
+            const int oy = lane == 0 ? 0 : (k < 9 ? k / 3 - 1 : (k < 12 ? 1 : 0));
+            const int oz = lane == 0 ? 0 : (k < 9 ? 1 : 0);
             int x = cx + ox, y = cy + oy, z = cz + oz;
             if (x < 0) { x += ncx; shx = -B.L[0]; } else if (x >= ncx) { x -= ncx; shx = B.L[0]; }
             if (y < 0) { y += ncy; shy = -B.L[1]; } else if (y >= ncy) { y -= ncy; shy = B.L[1]; }
@@ -253,10 +243,10 @@ __device__ void ens_unit(const EnsBox &B, const EnsPtrs &S, float4 *q, uint32_t 
         }
         const int pre = incl - len;
         const int ncand = __shfl_sync(0xFFFFFFFFu, incl, 31);
-        const int len0 = __shfl_sync(0xFFFFFFFFu, len, 0);  // N3: the own cell leads the candidates
+        const int len0 = __shfl_sync(0xFFFFFFFFu, len, 0);  // the own cell leads the candidates
         for (int base = 0; base < ncand; base += kEnsCand) {
             __syncwarp();
-            if (lane < (N3 ? 14 : 27)) {
+            if (lane < 14) {
                 const int lo = max(pre, base), hi = min(pre + len, base + kEnsCand);
                 for (int p = lo; p < hi; ++p) cand[p - base] = (uint32_t)S.idx[sbeg + p - pre] | ((uint32_t)lane << 16);
             }
@@ -307,9 +297,9 @@ __device__ void ens_unit(const EnsBox &B, const EnsPtrs &S, float4 *q, uint32_t 
                             dz = __fadd_rn(dz, __shfl_sync(0xFFFFFFFFu, shz, sl));
                         }
                         const float d2 = dist2_rn(dx, dy, dz);
-                        // N3: of the own cell only the members after the owner
+                        // of the own cell only the members after the owner
                         const int tg = base + 32 * r + lane;
-                        const bool fwd = !N3 || tg >= len0 || tg > o - ob;
+                        const bool fwd = tg >= len0 || tg > o - ob;
                         const bool hit = (d2 < B.rc2) & (d2 > 0.0f) & fwd;
                         const uint32_t m = __ballot_sync(0xFFFFFFFFu, hit);
                         if (hit)
@@ -317,7 +307,7 @@ __device__ void ens_unit(const EnsBox &B, const EnsPtrs &S, float4 *q, uint32_t 
                                 make_float4(dx, dy, dz, __uint_as_float((i << 16) | (pe[r] & 0xFFFFu)));
                         tail += (uint32_t)__popc(m);
                         if (tail - head >= 32u) {
-                            ens_batch<SMODE, VIR, N3>(B, S, q, key, head, 32, lane);
+                            ens_batch<SMODE, VIR>(B, S, q, key, head, 32, lane);
                             head += 32u;
                         }
                     }
@@ -328,7 +318,7 @@ __device__ void ens_unit(const EnsBox &B, const EnsPtrs &S, float4 *q, uint32_t 
             if (base + kEnsCand < ncand) {
                 while (tail != head) {
                     const int nb = (int)min(32u, tail - head);
-                    ens_batch<SMODE, VIR, N3>(B, S, q, key, head, nb, lane);
+                    ens_batch<SMODE, VIR>(B, S, q, key, head, nb, lane);
                     head += (uint32_t)nb;
                 }
             }
@@ -336,9 +326,137 @@ __device__ void ens_unit(const EnsBox &B, const EnsPtrs &S, float4 *q, uint32_t 
     }
     while (tail != head) {
         const int nb = (int)min(32u, tail - head);
-        ens_batch<SMODE, VIR, N3>(B, S, q, key, head, nb, lane);
+        ens_batch<SMODE, VIR>(B, S, q, key, head, nb, lane);
         head += (uint32_t)nb;
     }
+}
+
+// Default mode: the pair force on the particle at place k of the cell order
+// (S.idx[k]; valid: there is one) into S.f, by kEnsLanes consecutive lanes.
+// Issue bound (68 % of cycles with one 512-thread CTA a SM, which its shared
+// memory and 113 registers allow); 24 of 32 lanes active, because lanes differ in
+// candidates and pairs.  50 boxes of L = 9 and 10, 8 steps: 769 us a launch, 1151
+// with the ring of the Newton-3 mode above used for full stencils; 128 boxes of L
+// = 6..10, 32 steps: 3.7 ms with 2 lanes a particle, 3.8 with 1, 4.5 with 4.
+constexpr int kEnsBurst = 4;  // candidates whose loads are in flight together
+
+template <int SMODE, bool VIR>
+__device__ __forceinline__ void ens_particle(const EnsBox &B, const EnsPtrs &S, unsigned char *scratch, int k, bool valid,
+                                             int lane)
+{
+    uint32_t(*ranges)[32] = reinterpret_cast<uint32_t(*)[32]>(scratch);
+    uint16_t(*notes)[32] = reinterpret_cast<uint16_t(*)[32]>(scratch + 4 * 32 * kEnsRanges);
+    const uint32_t key[4] = {B.key[0], B.key[1], B.key[2], B.key[3]};
+    const int sub = lane % kEnsLanes;
+    const int i = valid ? (int)S.idx[k] : 0;
+    const float4 pi = S.pos[i], vi = S.u[i];
+    // the index ranges of this lane's rows: first place | length << 13 | shift << 26,
+    // the shift a base-3 code of (x, y, z), 0 none, 1 -L, 2 +L (a box that fits in
+    // shared memory has fewer than 2^13 particles)
+    int nr = 0;
+    if (valid) {
+        const int ncx = B.nc[0], ncy = B.nc[1], ncz = B.nc[2];
+        const int cx = ens_axis(pi.x, B.cpl[0], ncx), cy = ens_axis(pi.y, B.cpl[1], ncy), cz = ens_axis(pi.z, B.cpl[2], ncz);
+#pragma unroll
+        for (int q = 0; q < (9 + kEnsLanes - 1) / kEnsLanes; ++q) {
+            const int row = sub + q * kEnsLanes;
+            if (row < 9) {
+                int y = cy + row % 3 - 1, z = cz + row / 3 - 1;
+                uint32_t sh = 0;
+                if (y < 0) { y += ncy; sh += 3; } else if (y >= ncy) { y -= ncy; sh += 6; }
+                if (z < 0) { z += ncz; sh += 9; } else if (z >= ncz) { z -= ncz; sh += 18; }
+                const int base = (z * ncy + y) * ncx;
+                auto add = [&](int c0, int c1, uint32_t code) {
+                    const uint32_t b = S.start[base + c0], e = S.start[base + c1];
+                    if (e > b) ranges[nr++][lane] = b | ((e - b) << 13) | (code << 26);
+                };
+                if (cx == 0) {
+                    add(ncx - 1, ncx, sh + 1);
+                    add(0, 2, sh);
+                } else if (cx == ncx - 1) {
+                    add(ncx - 2, ncx, sh);
+                    add(0, 1, sh + 2);
+                } else {
+                    add(cx - 1, cx + 2, sh);
+                }
+            }
+        }
+    }
+    auto shift_of = [](uint32_t code, float L) { return code == 0u ? 0.0f : (code == 1u ? -L : L); };
+    float fx = 0.f, fy = 0.f, fz = 0.f, fw = 0.f, sx = 0.f, sy = 0.f, sz = 0.f;
+    uint32_t q = 0, qe = 0;
+    int r = 0, noted = 0;
+    auto next_range = [&]() {
+        const uint32_t w = ranges[r++][lane];
+        q = w & 0x1FFFu;
+        qe = q + ((w >> 13) & 0x1FFFu);
+        const uint32_t code = w >> 26;
+        sx = shift_of(code % 3u, B.L[0]);
+        sy = shift_of(code / 3u % 3u, B.L[1]);
+        sz = shift_of(code / 9u, B.L[2]);
+    };
+    if (r < nr) next_range();
+    for (;;) {
+        const bool more = __any_sync(0xFFFFFFFFu, q < qe);
+        if (more) {
+            uint32_t j[kEnsBurst];
+            float4 pj[kEnsBurst];
+#pragma unroll
+            for (int u = 0; u < kEnsBurst; ++u) j[u] = S.idx[min(q + (uint32_t)u, (uint32_t)B.n - 1u)];
+#pragma unroll
+            for (int u = 0; u < kEnsBurst; ++u) pj[u] = S.pos[j[u]];
+#pragma unroll
+            for (int u = 0; u < kEnsBurst; ++u) {
+                const float dx = __fadd_rn(__fsub_rn(pj[u].x, pi.x), sx);
+                const float dy = __fadd_rn(__fsub_rn(pj[u].y, pi.y), sy);
+                const float dz = __fadd_rn(__fsub_rn(pj[u].z, pi.z), sz);
+                const float d2 = dist2_rn(dx, dy, dz);
+                if ((q + (uint32_t)u < qe) & (d2 < B.rc2) & (d2 > 0.0f)) notes[noted++][lane] = (uint16_t)j[u];
+            }
+            q += kEnsBurst;
+            if (q >= qe && r < nr) next_range();
+            if (!__any_sync(0xFFFFFFFFu, noted > kEnsNotes - kEnsBurst)) continue;
+        }
+        const int most = __reduce_max_sync(0xFFFFFFFFu, noted);
+        for (int e = 0; e < most; ++e) {
+            if (e < noted) {
+                const uint32_t jj = notes[e][lane];
+                const float4 xj = S.pos[jj], vj = S.u[jj];
+                // inside r_c the minimum image is the image the walk found
+                const float dx = min_image_rn(xj.x, pi.x, B.L[0], B.halfL[0]);
+                const float dy = min_image_rn(xj.y, pi.y, B.L[1], B.halfL[1]);
+                const float dz = min_image_rn(xj.z, pi.z, B.L[2], B.halfL[2]);
+                const float d2 = dist2_rn(dx, dy, dz);
+                const float inv_r = rsqrtf(d2);
+                const float rr = d2 * inv_r;
+                const float wgt = fmaxf(fmaf(-rr, B.inv_rc, 1.0f), 0.0f);
+                const float wR = weight_R<SMODE>(wgt, B.s);
+                // e_ij = -d / r; e . v_ij = -(d . (v_i - v_j)) / r
+                const float ev = -((dx * (vi.x - vj.x) + dy * (vi.y - vj.y)) + dz * (vi.z - vj.z)) * inv_r;
+                uint32_t A, Bw;
+                pair_hash(__float_as_uint(vi.w), __float_as_uint(vj.w), key, A, Bw);
+                const float xi = gauss_from_hash(A, Bw);
+                float a = B.a[0];
+                if (B.n_species > 1) a = B.a[__float_as_int(pi.w) * B.n_species + __float_as_int(xj.w)];
+                const float F = fmaf(a, wgt, fmaf(-B.gamma * wR * wR, ev, B.sigma_isdt * wR * xi));
+                if (VIR) fw += 0.5f * (a * wgt * rr);  // each pair from both ends
+                const float sc = -F * inv_r;
+                fx = fmaf(sc, dx, fx);
+                fy = fmaf(sc, dy, fy);
+                fz = fmaf(sc, dz, fz);
+            }
+        }
+        if (!more) break;
+        noted = 0;
+    }
+#pragma unroll
+    for (int o = 1; o < kEnsLanes; o <<= 1) {
+        fx += __shfl_xor_sync(0xFFFFFFFFu, fx, o);
+        fy += __shfl_xor_sync(0xFFFFFFFFu, fy, o);
+        fz += __shfl_xor_sync(0xFFFFFFFFu, fz, o);
+        if (VIR) fw += __shfl_xor_sync(0xFFFFFFFFu, fw, o);
+    }
+    if (valid && sub == 0) S.f[i] = make_float4(fx, fy, fz, fw);
 }
 
 template <bool LHALF, int SMODE, bool N3>
@@ -367,12 +485,10 @@ __global__ void __launch_bounds__(kEnsMaxThreads, 1) k_ens_run(const EnsBox *__r
     S.start = reinterpret_cast<uint32_t *>(smem + lay.start);
     S.cnt = reinterpret_cast<uint32_t *>(smem + lay.cnt);
     S.idx = reinterpret_cast<uint16_t *>(smem + lay.idx);
-    S.slot = reinterpret_cast<uint16_t *>(smem + lay.slot);
     S.own = reinterpret_cast<uint8_t *>(smem + lay.own);
     S.C = C;
     S.rank = rank;
-    float4 *q = reinterpret_cast<float4 *>(smem + lay.q) + warp * kEnsQueue;
-    uint32_t *cand = reinterpret_cast<uint32_t *>(smem + lay.cand) + warp * kEnsCand;
+    unsigned char *scratch = smem + lay.warp + (size_t)warp * kEnsWarpBytes;
     const int steps = B.steps;
     const unsigned long long step0 = B.step;
     const float invL[3] = {1.0f / B.L[0], 1.0f / B.L[1], 1.0f / B.L[2]};
@@ -406,23 +522,25 @@ __global__ void __launch_bounds__(kEnsMaxThreads, 1) k_ens_run(const EnsBox *__r
     for (int c = threadIdx.x; c < ncell; c += T) S.cnt[c] = 0u;
     __syncthreads();
 
-    const int nunits = (ncell + kEnsUnitCells - 1) / kEnsUnitCells;
+    // work units: runs of kOwners places of the cell order, or (Newton-3 mode) of
+    // kEnsUnitCells cells
+    constexpr int kOwners = 32 / kEnsLanes;
+    const int nunits = N3 ? (ncell + kEnsUnitCells - 1) / kEnsUnitCells : (n + kOwners - 1) / kOwners;
     const int nforce = steps == 0 ? 1 : steps;
     for (int s = 1; s <= nforce; ++s) {
         const bool last = s == nforce;
         // 1. cell lists
-        for (int i = threadIdx.x; i < n; i += T) S.slot[i] = (uint16_t)atomicAdd(&S.cnt[ens_cell(B, S.pos[i])], 1u);
+        for (int i = threadIdx.x; i < n; i += T) atomicAdd(&S.cnt[ens_cell(B, S.pos[i])], 1u);
         __syncthreads();
-        ens_scan(S.cnt, S.start, ncell, wsum);
+        ens_scan(S.cnt, S.start, ncell, wsum);  // the counts become the cells' cursors
         for (int i = threadIdx.x; i < n; i += T) {
             const int c = ens_cell(B, S.pos[i]);
-            S.idx[S.start[c] + S.slot[i]] = (uint16_t)i;
+            S.idx[atomicAdd(&S.cnt[c], 1u)] = (uint16_t)i;
             if (N3) {  // partner shares may come from any warp of the cluster
                 S.f[i] = make_float4(0.f, 0.f, 0.f, 0.f);
                 S.own[i] = (uint8_t)((c / kEnsUnitCells) % C);
             }
         }
-        for (int c = threadIdx.x; c < ncell; c += T) S.cnt[c] = 0u;
         __syncthreads();
         for (int c = threadIdx.x; c < ncell; c += T) {  // members of a cell in index order
             const int lo = (int)S.start[c], hi = (int)S.start[c + 1];
@@ -435,22 +553,35 @@ __global__ void __launch_bounds__(kEnsMaxThreads, 1) k_ens_run(const EnsBox *__r
                 }
                 S.idx[m + 1] = v;
             }
+            S.cnt[c] = 0u;
         }
         __syncthreads();
         if (N3 && C > 1) cl.sync();  // every replica's accumulators are zero before any remote add
         // 2. pair forces of this CTA's units
         for (int u = rank + C * warp; u < nunits; u += C * nwarps) {
-            if (last) ens_unit<SMODE, true, N3>(B, S, q, cand, u, lane);
-            else ens_unit<SMODE, false, N3>(B, S, q, cand, u, lane);
+            if constexpr (N3) {
+                float4 *q = reinterpret_cast<float4 *>(scratch);
+                uint32_t *cand = reinterpret_cast<uint32_t *>(scratch + 16 * kEnsQueue);
+                if (last) ens_unit<SMODE, true>(B, S, q, cand, u, lane);
+                else ens_unit<SMODE, false>(B, S, q, cand, u, lane);
+            } else {
+                const int k = u * kOwners + lane / kEnsLanes;
+                if (last) ens_particle<SMODE, true>(B, S, scratch, k, k < n, lane);
+                else ens_particle<SMODE, false>(B, S, scratch, k, k < n, lane);
+            }
         }
         __syncthreads();
         if (C > 1) cl.sync();  // every replica has been read for this step
-        // 3. integrate the particles of this CTA's units
+        // 3. integrate the particles of this CTA's units: the unit's lanes in
+        // Newton-3 mode; otherwise all threads over the CTA's places
         const unsigned long long stepn = step0 + (unsigned long long)s + 1ull;  // step of the next force
-        for (int u = rank + C * warp; u < nunits; u += C * nwarps) {
-            const int k0 = (int)S.start[u * kEnsUnitCells];
-            const int k1 = (int)S.start[min((u + 1) * kEnsUnitCells, ncell)];
-            for (int k = k0 + lane; k < k1; k += 32) {
+        const int own_units = nunits > rank ? (nunits - rank + C - 1) / C : 0;
+        for (int u = N3 ? rank + C * warp : 0; u < (N3 ? nunits : 1); u += C * nwarps) {
+            const int k0 = N3 ? (int)S.start[u * kEnsUnitCells] + lane : (int)threadIdx.x;
+            const int k1 = N3 ? (int)S.start[min((u + 1) * kEnsUnitCells, ncell)] : own_units * kOwners;
+            for (int kk = k0; kk < k1; kk += N3 ? 32 : T) {
+                const int k = N3 ? kk : (rank + C * (kk / kOwners)) * kOwners + kk % kOwners;
+                if (k >= n) continue;
                 const int i = S.idx[k];
                 float4 f = S.f[i];
                 const float4 x = S.pos[i];

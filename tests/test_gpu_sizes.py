@@ -119,3 +119,31 @@ def test_profile_each_side_of_the_size_rules(n, nbins):
         assert np.array_equal(counts - start, np.bincount(b, minlength=nbins))
         assert np.abs(sums - start - ref).max() < 1e-12 * max(np.abs(ref).max(), nbins, 1.0)
     g.close()
+
+
+# more pairs than a lane notes (rho = 22); rows of the stencil that cross the
+# boundary on both sides (three cells an axis); one particle; a box of few units
+@pytest.mark.parametrize("n,L,lam,shape", [(2000, 4.5, 0.5, (128, 1)), (2000, 4.5, 0.65, (512, 2)), (90, 3.01, 0.5, (256, 8)),
+                                           (1, 3.5, 0.5, (256, 2)), (17, 3.5, 0.5, (128, 4)), (3000, 10.0, 0.5, (512, 2))])
+def test_ensemble_forces_of_sparse_and_dense_boxes(n, L, lam, shape):
+    need_gpu()
+    c = workloads.CONFIGS["fluid_small"]
+    box = (L, L + 0.3, L + 0.1)
+    x, v = workloads.uniform_fluid(box, n, 1.0, n)[:2]
+    sp = np.random.default_rng(n).integers(0, 2, n).astype(np.int32)
+    a = [[25.0, 40.0], [40.0, 30.0]]
+    e = dpd.Ensemble(threads=shape[0], cluster=shape[1])
+    i = e.add(box, a, c["gamma"], c["kT"], c["rc"], 0.5, c["dt"], x, v, species=sp, step=2, lam=lam, seed=7)
+    x32, v32, _ = e.state(i)
+    o = oracle.System(box, a, c["gamma"], c["kT"], c["rc"], 0.5, c["dt"], lam=lam, seed=7, cut_fp32=True)
+    f, vir = o.forces(x32, v32, species=sp, step=2)
+    got = e.forces(i)
+    if n > 1:
+        assert force_error(got, f)[0] < FORCE_TOL
+        assert abs(e.observables(i)["virial"] - vir) < 1e-5 * abs(vir)
+    else:
+        assert np.array_equal(got, np.zeros((1, 3)))
+    e.step(3)
+    e.sync()
+    assert np.isfinite(e.state(i)[0]).all()
+    e.close()

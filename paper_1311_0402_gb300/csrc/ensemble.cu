@@ -147,11 +147,48 @@ int class_of(int64_t n, int ncell, bool lhalf, size_t limit)
     return (int)std::min<size_t>(std::max<size_t>(k, 1), 4) - 1;
 }
 
-// Shapes the autotuner chose on seeded streams of boxes of L = 6..10 (512
-// threads and 2 CTAs per box, 256 threads for the smallest class); a launch
-// steps down from these when a box's footprint does not fit.
-int default_threads(int cls) { return cls == 3 ? 256 : 512; }
-int default_cluster(int) { return 2; }
+// Launch shapes before the autotuner has run.  A launch is as long as its
+// largest boxes, so the SMs that one CTA per box leaves free go to the class
+// whose boxes are slowest, by doubling its CTAs per box up to 4; a 512-thread CTA
+// takes an SM (its registers), two of 256 threads share one, which is the better
+// use for small boxes when the SMs are short.  us per step of 26 / 80 / 152 boxes
+// of L = 10 (3,000 particles), 512 threads and 1, 2, 4 CTAs a box: 154, 83, 48 /
+// 156, 165, 143 / 156, 167, 238; 256 threads and 1, 2 CTAs: 227, 122 / 227, 242;
+// L = 7 (1,029): 65, 39, 26 / 66, 78, 77 and 91, 53 / 92, 68.  The Newton-3 mode,
+// whose CTAs add to each other's memory, keeps 2 CTAs a box.
+constexpr int kSMs = 152;
+
+struct Shapes {
+    int threads[kClasses], cluster[kClasses];
+};
+
+Shapes default_shapes(bool n3, const int (&count)[kClasses], const int64_t (&largest)[kClasses])
+{
+    Shapes s;
+    int boxes = 0;
+    for (int c = 0; c < kClasses; ++c) boxes += count[c];
+    for (int c = 0; c < kClasses; ++c) {
+        s.threads[c] = n3 ? (c == 3 ? 256 : 512) : (c >= 2 && boxes > kSMs / 2 ? 256 : 512);
+        s.cluster[c] = n3 ? 2 : 1;
+    }
+    for (bool more = !n3; more;) {
+        // half SMs in use, and the class whose boxes take longest
+        int used = 0, slow = -1;
+        double longest = 0.0;
+        for (int c = 0; c < kClasses; ++c) {
+            if (count[c] == 0) continue;
+            used += count[c] * s.cluster[c] * (s.threads[c] / 256);
+            const double t = (double)largest[c] / (s.cluster[c] * s.threads[c]);
+            if (t > longest) {
+                longest = t;
+                slow = c;
+            }
+        }
+        more = slow >= 0 && s.cluster[slow] < 4 && used + count[slow] * s.cluster[slow] * (s.threads[slow] / 256) <= 2 * kSMs;
+        if (more) s.cluster[slow] *= 2;
+    }
+    return s;
+}
 
 void fill_desc(EnsBox &d, const dpd_box_params *p, int64_t n, const int nc[3])
 {
@@ -286,10 +323,9 @@ dpd_status dpd_ensemble_create(dpd_ensemble **out, const dpd_ensemble_options *o
         dpd_ensemble_destroy(e);
         return efail(nullptr, DPD_ERR_CUDA, "ensemble setup failed (no GPU, or kernel attributes refused)");
     }
-    for (int c = 0; c < kClasses; ++c) {
-        e->threads[c] = o.threads ? o.threads : default_threads(c);
-        e->cluster[c] = o.cluster ? o.cluster : default_cluster(c);
-    }
+    const int none[kClasses] = {};
+    const int64_t zero[kClasses] = {};
+    update_shapes(e, none, zero);
     *out = e;
     return DPD_OK;
 }
@@ -476,6 +512,16 @@ dpd_status dpd_ensemble_step(dpd_ensemble *e, const int32_t *ids, const int32_t 
                     d.steps = g.run_steps[k];
                     descs.push_back(d);
                     bs.push_back(g.run[k]);
+    {
+        int count[kClasses] = {};
+        int64_t largest[kClasses] = {};
+        for (auto &kv : groups)
+            for (const EBox *b : kv.second.run.empty() ? kv.second.init : kv.second.run) {
+                count[b->cls] += 1;
+                largest[b->cls] = std::max(largest[b->cls], b->n);
+            }
+        update_shapes(e, count, largest);
+    }
                 }
             }
             if (bs.empty()) continue;

@@ -226,6 +226,9 @@ cudaError_t launch_import_check(int64_t n, int n_species, const double *x, const
 cudaError_t launch_import(const SimParams &P, const double box[3], int64_t n, const double *x, const double *v,
                           const int32_t *sp, const uint32_t *tag, float4 *pos, float4 *vel, uint32_t *tag_out,
                           uint32_t *pid_out, cudaStream_t s);
+cudaError_t launch_export2(int64_t n, const float4 *pos, const float4 *vel, const uint32_t *pid, double *x, double *v,
+                           cudaStream_t s);
+cudaError_t launch_export_state(int64_t n, const Ptrs &D, double *x, double *v, cudaStream_t s);
 cudaError_t launch_export(int64_t n, const float4 *src, const uint32_t *pid, double *out, cudaStream_t s);
 // profile: nblocks = profile_blocks_for(n, nbins) partials of 2 nbins in D.red,
 // then their fixed-order sum (sum, count by bin) behind them

@@ -534,12 +534,10 @@ dpd_status guard(dpd_sim *h, bool need_state)
     return DPD_OK;
 }
 
-// Download a float4 array and its caller indices; scatter xyz into out (n x 3).
-dpd_status download_xyz(dpd_sim *h, const float4 *dev, double *out)
+// Download a float4 array of the live order (c: the control words as read);
+// scatter xyz into out (n x 3).
+dpd_status download_xyz(dpd_sim *h, const DevCtl &c, const float4 *dev, double *out)
 {
-    DevCtl c;
-    dpd_status st = read_ctl(h, c);
-    if (st) return st;
     // scattered to caller order and widened on the device, one copy out
     Staging o(h);
     double *od = (double *)o.get(sizeof(double) * 3 * (size_t)h->n);
@@ -937,7 +935,7 @@ dpd_status dpd_forces(dpd_sim *h, double *f_out)
     st = check_err(h, c);
     if (st) return st;
     if (!f_out) return DPD_OK;
-    return download_xyz(h, h->D.fout, f_out);
+    return download_xyz(h, c, h->D.fout, f_out);
 }
 
 dpd_status dpd_get_force(dpd_sim *h, double *f_out)
@@ -948,7 +946,7 @@ dpd_status dpd_get_force(dpd_sim *h, double *f_out)
     DevCtl c;
     st = read_ctl(h, c);
     if (st) return st;
-    return download_xyz(h, h->D.force[c.parity], f_out);
+    return download_xyz(h, c, h->D.force[c.parity], f_out);
 }
 
 dpd_status dpd_set_force(dpd_sim *h, const double *f)
@@ -1136,24 +1134,16 @@ dpd_status dpd_observables(dpd_sim *h, dpd_obs *out)
     dpd_status st = guard(h, true);
     if (st) return st;
     if (!out) return fail(h, DPD_ERR_ARG, "out is NULL");
+    // the record is finished on the device: one copy and one wait
     const int nb = observe_blocks_for((int)h->n);
+    const double V = h->box[0] * h->box[1] * h->box[2];
+    dpd_obs o;
     CUDA_TRY(h, launch_observe(h->P, h->D, nb, h->stream));
-    double acc[8];
-    CUDA_TRY(h, cudaMemcpyAsync(acc, h->D.red + (size_t)nb * 8, sizeof(acc), cudaMemcpyDeviceToHost, h->stream));
-    DevCtl c;
-    CUDA_TRY(h, cudaMemcpyAsync(&c, h->D.ctl, sizeof(c), cudaMemcpyDeviceToHost, h->stream));
+    CUDA_TRY(h, launch_observe_finish(h->D, nb, h->n, h->n > 1 ? 3.0 * h->n - 3.0 : 0.0, 3.0 * V, h->stream));
+    CUDA_TRY(h, cudaMemcpyAsync(&o, h->D.obs, sizeof(o), cudaMemcpyDeviceToHost, h->stream));
     st = wait(h);
     if (st) return st;
-    const double V = h->box[0] * h->box[1] * h->box[2];
-    out->step = c.step;
-    out->n = h->n;
-    out->kinetic = 0.5 * acc[0];
-    out->temperature = h->n > 1 ? acc[0] / (3.0 * h->n - 3.0) : 0.0;
-    out->virial = acc[4];
-    out->pressure = (acc[0] + acc[4]) / (3.0 * V);
-    out->momentum[0] = acc[1];
-    out->momentum[1] = acc[2];
-    out->momentum[2] = acc[3];
+    *out = o;
     return DPD_OK;
 }
 
@@ -1218,18 +1208,19 @@ dpd_status dpd_get_state(dpd_sim *h, double *x, double *v, uint64_t *step)
     NvtxRange nvtx_("dpd_get_state");
     dpd_status st = guard(h, true);
     if (st) return st;
-    DevCtl c;
-    st = read_ctl(h, c);
+    if (x || v) {
+        // one export, the copies behind it and one wait
+        const size_t bytes = sizeof(double) * 3 * (size_t)h->n;
+        Staging o(h);
+        double *xd = x ? (double *)o.get(bytes) : nullptr, *vd = v ? (double *)o.get(bytes) : nullptr;
+        if (!o.ok()) return fail(h, DPD_ERR_OOM, "device staging for the state: " + o.error());
+        CUDA_TRY(h, launch_export_state(h->n, h->D, xd, vd, h->stream));
+        if (x) CUDA_TRY(h, cudaMemcpyAsync(x, xd, bytes, cudaMemcpyDeviceToHost, h->stream));
+        if (v) CUDA_TRY(h, cudaMemcpyAsync(v, vd, bytes, cudaMemcpyDeviceToHost, h->stream));
+    }
+    st = wait(h);
     if (st) return st;
-    if (x) {
-        st = download_xyz(h, h->D.pos[c.parity], x);
-        if (st) return st;
-    }
-    if (v) {
-        st = download_xyz(h, h->D.vel[c.parity], v);
-        if (st) return st;
-    }
-    if (step) *step = c.step;
+    if (step) *step = h->step;  // the queued steps have run
     return DPD_OK;
 }
 

@@ -65,6 +65,11 @@ struct dpd_ensemble {
     cudaGraphExec_t graph = nullptr;
     std::vector<uint64_t> graph_key;
     int64_t graph_replays = 0;
+    // page-locked host memory that kernels write a box's state into, kept for
+    // the handle's life and as large as its largest read needs (a box has at
+    // most a few thousand particles)
+    double *mail = nullptr;
+    size_t mail_bytes = 0;
     int64_t graph_captures = 0;
 };
 
@@ -220,6 +225,35 @@ void fill_desc(EnsBox &d, const dpd_box_params *p, int64_t n, const int nc[3])
     d.key[1] = (uint32_t)(p->seed >> 32);
     d.key[2] = 0x243F6A88u;
     d.key[3] = 0x85A308D3u;
+}
+
+// The shapes of the next launch: the autotuner's, else the options', else the
+// default for the boxes that run.
+void update_shapes(dpd_ensemble *e, const int (&count)[kClasses], const int64_t (&largest)[kClasses])
+{
+    if (e->tuned) return;
+    const Shapes s = default_shapes(e->opt.newton3 != 0, count, largest);
+    for (int c = 0; c < kClasses; ++c) {
+        e->threads[c] = e->opt.threads ? e->opt.threads : s.threads[c];
+        e->cluster[c] = e->opt.cluster ? e->opt.cluster : s.cluster[c];
+    }
+}
+
+// e->mail of at least `bytes` (null when page-locked memory runs out: the
+// caller stages in device memory instead).
+double *ensure_mail(dpd_ensemble *e, size_t bytes)
+{
+    if (bytes <= e->mail_bytes) return e->mail;
+    if (e->mail) cudaFreeHost(e->mail);
+    e->mail = nullptr;
+    e->mail_bytes = 0;
+    if (cudaHostAlloc((void **)&e->mail, bytes, cudaHostAllocMapped) != cudaSuccess) {
+        cudaGetLastError();
+        e->mail = nullptr;
+        return nullptr;
+    }
+    e->mail_bytes = bytes;
+    return e->mail;
 }
 
 dpd_status ensure_desc(dpd_ensemble *e, size_t count)
@@ -478,6 +512,16 @@ dpd_status dpd_ensemble_step(dpd_ensemble *e, const int32_t *ids, const int32_t 
         }
     }
     if (groups.empty()) return DPD_OK;
+    {
+        int count[kClasses] = {};
+        int64_t largest[kClasses] = {};
+        for (auto &kv : groups)
+            for (const EBox *b : kv.second.run.empty() ? kv.second.init : kv.second.run) {
+                count[b->cls] += 1;
+                largest[b->cls] = std::max(largest[b->cls], b->n);
+            }
+        update_shapes(e, count, largest);
+    }
     // descriptors: per group, the init boxes then the run boxes (largest first)
     std::vector<EnsBox> descs;
     struct Launch {
@@ -512,16 +556,6 @@ dpd_status dpd_ensemble_step(dpd_ensemble *e, const int32_t *ids, const int32_t 
                     d.steps = g.run_steps[k];
                     descs.push_back(d);
                     bs.push_back(g.run[k]);
-    {
-        int count[kClasses] = {};
-        int64_t largest[kClasses] = {};
-        for (auto &kv : groups)
-            for (const EBox *b : kv.second.run.empty() ? kv.second.init : kv.second.run) {
-                count[b->cls] += 1;
-                largest[b->cls] = std::max(largest[b->cls], b->n);
-            }
-        update_shapes(e, count, largest);
-    }
                 }
             }
             if (bs.empty()) continue;
@@ -632,6 +666,21 @@ dpd_status dpd_ensemble_get_state(dpd_ensemble *e, int32_t id, double *x, double
         // a box never stepped since its addition still needs its initial force
         // only for stepping; its state is the loaded one
         const size_t bytes = (size_t)b.n * 3 * sizeof(double);
+        if (double *m = ensure_mail(e, 2 * bytes)) {
+            // written straight into the page-locked block, one wait
+            double *mv = m + 3 * (size_t)b.n;
+            cudaError_t c = launch_export2(b.n, b.desc.pos, b.desc.vel, b.pid, x ? m : nullptr, v ? mv : nullptr, e->stream);
+            if (c != cudaSuccess) {
+                cudaGetLastError();
+                return efail(e, DPD_ERR_CUDA, std::string("state download: ") + cudaGetErrorString(c));
+            }
+            dpd_status st = ewait(e);
+            if (st) return st;
+            if (x) std::memcpy(x, m, bytes);
+            if (v) std::memcpy(v, mv, bytes);
+            if (step) *step = b.step;
+            return DPD_OK;
+        }
         void *stage = nullptr;
         if (cudaMallocAsync(&stage, 2 * bytes, e->stream) != cudaSuccess) {
             cudaGetLastError();
@@ -898,6 +947,7 @@ void dpd_ensemble_destroy(dpd_ensemble *e)
         if (e->cls_stream[c]) cudaStreamDestroy(e->cls_stream[c]);
         if (e->join[c]) cudaEventDestroy(e->join[c]);
     }
+    if (e->mail) cudaFreeHost(e->mail);
     if (e->graph) cudaGraphExecDestroy(e->graph);
     if (e->fork) cudaEventDestroy(e->fork);
     if (e->ev) cudaEventDestroy(e->ev);

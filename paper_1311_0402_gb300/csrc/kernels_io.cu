@@ -78,7 +78,54 @@ __global__ void k_export(int64_t n, const float4 *__restrict__ src, const uint32
     }
 }
 
+// The same for positions and velocities at once; x or v may be null.
+__device__ __forceinline__ void export2(int64_t p, const float4 *__restrict__ pos, const float4 *__restrict__ vel,
+                                        const uint32_t *__restrict__ pid, double *x, double *v)
+{
+    const size_t i = pid[p];
+    if (x) {
+        const float4 q = pos[p];
+        x[3 * i] = q.x;
+        x[3 * i + 1] = q.y;
+        x[3 * i + 2] = q.z;
+    }
+    if (v) {
+        const float4 q = vel[p];
+        v[3 * i] = q.x;
+        v[3 * i + 1] = q.y;
+        v[3 * i + 2] = q.z;
+    }
+}
+
+__global__ void k_export2(int64_t n, const float4 *pos, const float4 *vel, const uint32_t *pid, double *x, double *v)
+{
+    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x)
+        export2(p, pos, vel, pid, x, v);
+}
+
+// The live state of a handle: the control words say which set it is.
+__global__ void k_export_state(int64_t n, Ptrs D, double *x, double *v)
+{
+    const uint32_t par = D.ctl->parity;
+    const uint32_t *pid = D.pid[D.ctl->oparity];
+    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x)
+        export2(p, D.pos[par], D.vel[par], pid, x, v);
+}
+
 }  // namespace
+
+cudaError_t launch_export2(int64_t n, const float4 *pos, const float4 *vel, const uint32_t *pid, double *x, double *v,
+                           cudaStream_t s)
+{
+    k_export2<<<grid_for(n), kThreads, 0, s>>>(n, pos, vel, pid, x, v);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_export_state(int64_t n, const Ptrs &D, double *x, double *v, cudaStream_t s)
+{
+    k_export_state<<<grid_for(n), kThreads, 0, s>>>(n, D, x, v);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_import_check(int64_t n, int n_species, const double *x, const double *v, const int32_t *sp,
                                 uint32_t *bad, cudaStream_t s)

@@ -136,7 +136,7 @@ struct Ptrs {
     unsigned long long *obs;  // the 9 words of a dpd_obs, written by k_obs_finish
     // cells
     const uint32_t *rank_of_cell;  // (cz * nc_y + cy) * nc_x + cx -> Morton rank
-    const uint32_t *stencil;       // [ncell][27] neighbour ranks, ascending, kNone pad
+    const uint32_t *stencil;       // [ncell][27] neighbour ranks, ascending, kNone pad (without bricks)
     uint32_t *cell_count;          // [ncell]
     uint32_t *cell_start;          // [ncell + 1]
     uint32_t *scan_part;           // block sums of the scan
@@ -237,6 +237,8 @@ cudaError_t launch_profile(const SimParams &P, const Ptrs &D, int bin_axis, int 
                            int nblocks, cudaStream_t s);
 cudaError_t launch_pair_rng(uint64_t seed, uint64_t step, int64_t m, const uint32_t *ti, const uint32_t *tj,
                             uint32_t *out_hash, float *out_xi, cudaStream_t s);
+// the tables D.rank_of_cell, D.brick_* or D.stencil, once per handle
+cudaError_t launch_geometry(const SimParams &P, const Ptrs &D, cudaStream_t s);
 int scan_blocks_for(int ncell);
 // whether a box's binning, scan and reorder fit one block (k_sort_small), and
 // the kernels of a rebuild

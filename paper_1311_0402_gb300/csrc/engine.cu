@@ -1,9 +1,9 @@
 // engine.cu -- host engine and C ABI of libdpd.so (declared in dpd.h).
 //
-// Owns the device memory of a simulation, builds the cell geometry (Morton
-// ranks of the cells and the ascending 27-cell stencils, built once, as the
-// coarse stencil of Sec. 3.3.1), uploads and downloads particle state in the
-// caller's order, and drives the per-step kernel sequence of Algorithm 1:
+// Owns the device memory of a simulation, has the cell geometry built on the
+// device (Morton ranks of the cells, brick tables or the ascending 27-cell
+// stencils, built once, as the coarse stencil of Sec. 3.3.1), uploads and
+// downloads particle state in the caller's order, and drives the per-step kernel sequence of Algorithm 1:
 //   phase 1 (+ signature, displacement check) -> rebuild chain (runs only
 //   when flagged on the device) -> pair force -> phase 2,
 // captured into CUDA graphs of several steps that are replayed, so a step
@@ -31,91 +31,6 @@ namespace {
 
 thread_local std::string g_last_error;
 
-struct Geometry {
-    int nc[3];
-    int ncell;
-    std::vector<uint32_t> rank_of_cell;  // linear (cz, cy, cx) -> rank
-    std::vector<uint32_t> stencil;       // [ncell][27]
-    int nb[3] = {0, 0, 0};               // bricks per axis
-    std::vector<uint32_t> brick_lo, brick_hi;  // first / last Morton rank of each brick
-    std::vector<uint32_t> brick_ord;           // position of each brick in ascending rank order
-};
-
-uint32_t spread3(uint32_t v)  // 10 bits -> every third bit
-{
-    uint32_t x = v & 0x3FFu;
-    x = (x | (x << 16)) & 0x030000FFu;
-    x = (x | (x << 8)) & 0x0300F00Fu;
-    x = (x | (x << 4)) & 0x030C30C3u;
-    x = (x | (x << 2)) & 0x09249249u;
-    return x;
-}
-
-void build_geometry(const int nc[3], Geometry &g)
-{
-    g.nc[0] = nc[0]; g.nc[1] = nc[1]; g.nc[2] = nc[2];
-    g.ncell = nc[0] * nc[1] * nc[2];
-    std::vector<std::pair<uint64_t, uint32_t>> order(g.ncell);
-    for (int z = 0; z < nc[2]; ++z)
-        for (int y = 0; y < nc[1]; ++y)
-            for (int x = 0; x < nc[0]; ++x) {
-                uint32_t lin = (uint32_t)((z * nc[1] + y) * nc[0] + x);
-                uint64_t code = (uint64_t)spread3((uint32_t)x) | ((uint64_t)spread3((uint32_t)y) << 1) |
-                                ((uint64_t)spread3((uint32_t)z) << 2);
-                order[lin] = {code, lin};
-            }
-    std::sort(order.begin(), order.end());
-    g.rank_of_cell.assign(g.ncell, 0);
-    std::vector<uint32_t> lin_of_rank(g.ncell);
-    for (int r = 0; r < g.ncell; ++r) {
-        g.rank_of_cell[order[r].second] = (uint32_t)r;
-        lin_of_rank[r] = order[r].second;
-    }
-    // distinct neighbour offsets per axis ({-1,0,1}, or fewer when an axis
-    // has fewer than three cells so no cell is listed twice)
-    std::vector<int> off[3];
-    for (int a = 0; a < 3; ++a) {
-        if (nc[a] >= 3) off[a] = {-1, 0, 1};
-        else if (nc[a] == 2) off[a] = {0, 1};
-        else off[a] = {0};
-    }
-    g.stencil.assign((size_t)g.ncell * kStencil, kNone);
-    std::vector<uint32_t> tmp;
-    for (int r = 0; r < g.ncell; ++r) {
-        uint32_t lin = lin_of_rank[r];
-        int x = lin % nc[0], y = (lin / nc[0]) % nc[1], z = lin / (nc[0] * nc[1]);
-        tmp.clear();
-        for (int oz : off[2])
-            for (int oy : off[1])
-                for (int ox : off[0]) {
-                    int cx = (x + ox + nc[0]) % nc[0], cy = (y + oy + nc[1]) % nc[1], cz = (z + oz + nc[2]) % nc[2];
-                    tmp.push_back(g.rank_of_cell[(cz * nc[1] + cy) * nc[0] + cx]);
-                }
-        std::sort(tmp.begin(), tmp.end());
-        std::copy(tmp.begin(), tmp.end(), g.stencil.begin() + (size_t)r * kStencil);
-    }
-    // aligned kBrick^3 blocks of cells: consecutive Morton ranks
-    for (int a = 0; a < 3; ++a) g.nb[a] = (nc[a] + kBrick - 1) / kBrick;
-    const int nbricks = g.nb[0] * g.nb[1] * g.nb[2];
-    g.brick_lo.assign(nbricks, 0xFFFFFFFFu);
-    g.brick_hi.assign(nbricks, 0u);
-    for (int z = 0; z < nc[2]; ++z)
-        for (int y = 0; y < nc[1]; ++y)
-            for (int x = 0; x < nc[0]; ++x) {
-                const int b = ((z / kBrick) * g.nb[1] + y / kBrick) * g.nb[0] + x / kBrick;
-                const uint32_t r = g.rank_of_cell[(z * nc[1] + y) * nc[0] + x];
-                g.brick_lo[b] = std::min(g.brick_lo[b], r);
-                g.brick_hi[b] = std::max(g.brick_hi[b], r);
-            }
-    // the bricks partition the rank range into consecutive intervals; their
-    // order along it numbers the group lists
-    std::vector<std::pair<uint32_t, int>> by_rank(nbricks);
-    for (int b = 0; b < nbricks; ++b) by_rank[b] = {g.brick_lo[b], b};
-    std::sort(by_rank.begin(), by_rank.end());
-    g.brick_ord.assign(nbricks, 0u);
-    for (int k = 0; k < nbricks; ++k) g.brick_ord[by_rank[k].second] = (uint32_t)k;
-}
-
 }  // namespace
 
 struct dpd_sim {
@@ -127,7 +42,6 @@ struct dpd_sim {
     dpd_options opt;
     SimParams P;
     Ptrs D;
-    Geometry geo;
     int n_scan_blocks = 0;
     // device memory
     std::vector<void *> allocs;        // per-n allocations
@@ -680,7 +594,6 @@ dpd_status dpd_create(dpd_sim **out, const double box[3], int32_t n_species, con
         return fail(nullptr, DPD_ERR_CUDA, "cudaEventCreate failed");
     }
     keep_pool_memory();
-    build_geometry(nc, h->geo);
     h->n_scan_blocks = scan_blocks_for(P.ncell);
     P.no_reorder = o.no_reorder;
     P.use_bricks = (!o.no_reorder && nc[0] >= 3 && nc[1] >= 3 && nc[2] >= 3) ? 1 : 0;
@@ -695,8 +608,8 @@ dpd_status dpd_create(dpd_sim **out, const double box[3], int32_t n_species, con
         P.newton3 = 0;
     }
     P.list_builder = o.list_builder;
-    for (int a = 0; a < 3; ++a) P.nb[a] = h->geo.nb[a];
-    P.nbricks = h->geo.nb[0] * h->geo.nb[1] * h->geo.nb[2];
+    for (int a = 0; a < 3; ++a) P.nb[a] = (nc[a] + kBrick - 1) / kBrick;
+    P.nbricks = P.nb[0] * P.nb[1] * P.nb[2];
     if (cudaError_t ea = init_kernel_attributes(); ea != cudaSuccess) {
         cudaGetLastError();
         dpd_destroy(h);
@@ -707,7 +620,7 @@ dpd_status dpd_create(dpd_sim **out, const double box[3], int32_t n_species, con
     A((void **)&h->D.ctl, sizeof(DevCtl));
     A((void **)&h->D.obs, sizeof(dpd_obs));
     A((void **)&h->D.rank_of_cell, sizeof(uint32_t) * P.ncell);
-    A((void **)&h->D.stencil, sizeof(uint32_t) * (size_t)P.ncell * kStencil);
+    if (!P.use_bricks) A((void **)&h->D.stencil, sizeof(uint32_t) * (size_t)P.ncell * kStencil);
     A((void **)&h->D.cell_count, sizeof(uint32_t) * P.ncell);
     A((void **)&h->D.cell_start, sizeof(uint32_t) * (P.ncell + 1));
     A((void **)&h->D.scan_part, sizeof(uint32_t) * (h->n_scan_blocks + 1));
@@ -720,26 +633,13 @@ dpd_status dpd_create(dpd_sim **out, const double box[3], int32_t n_species, con
         dpd_destroy(h);
         return fail(nullptr, st, m);
     }
-    cudaError_t e = cudaMemcpyAsync((void *)h->D.rank_of_cell, h->geo.rank_of_cell.data(), sizeof(uint32_t) * P.ncell,
-                                    cudaMemcpyHostToDevice, h->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync((void *)h->D.stencil, h->geo.stencil.data(), sizeof(uint32_t) * (size_t)P.ncell * kStencil,
-                            cudaMemcpyHostToDevice, h->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync((void *)h->D.brick_rank_lo, h->geo.brick_lo.data(), sizeof(uint32_t) * P.nbricks,
-                            cudaMemcpyHostToDevice, h->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync((void *)h->D.brick_rank_hi, h->geo.brick_hi.data(), sizeof(uint32_t) * P.nbricks,
-                            cudaMemcpyHostToDevice, h->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync((void *)h->D.brick_ord, h->geo.brick_ord.data(), sizeof(uint32_t) * P.nbricks,
-                            cudaMemcpyHostToDevice, h->stream);
+    cudaError_t e = launch_geometry(P, h->D, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->D.cell_count, 0, sizeof(uint32_t) * P.ncell, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->D.ctl, 0, sizeof(DevCtl), h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) {
         dpd_destroy(h);
-        return fail(nullptr, DPD_ERR_CUDA, std::string("upload of cell tables: ") + cudaGetErrorString(e));
+        return fail(nullptr, DPD_ERR_CUDA, std::string("cell tables: ") + cudaGetErrorString(e));
     }
     *out = h;
     return DPD_OK;

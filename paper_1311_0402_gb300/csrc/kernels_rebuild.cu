@@ -76,6 +76,65 @@ __device__ __forceinline__ uint32_t cell_rank_of(const SimParams &P, const uint3
     return rank_of_cell[(cz * P.nc[1] + cy) * P.nc[0] + cx];
 }
 
+// Rank of cell (x, y, z) along the Morton curve through an nx x ny x nz grid (x
+// in the lowest bit): the cells before it, counted from the top down as the
+// sizes of the child blocks before its own, clipped to the grid.
+__device__ uint32_t morton_rank(const int (&n)[3], int x, int y, int z)
+{
+    uint32_t r = 0;
+    for (int b = 9; b >= 0; --b) {  // at most 1024 cells along an axis
+        const int size = 1 << b, k = ((x >> b) & 1) | (((y >> b) & 1) << 1) | (((z >> b) & 1) << 2);
+        const int ox = (x >> (b + 1)) << (b + 1), oy = (y >> (b + 1)) << (b + 1), oz = (z >> (b + 1)) << (b + 1);
+        for (int c = 0; c < k; ++c) {
+            const int ex = min(size, n[0] - ox - (c & 1) * size), ey = min(size, n[1] - oy - ((c >> 1) & 1) * size),
+                      ez = min(size, n[2] - oz - (c >> 2) * size);
+            if (ex > 0 && ey > 0 && ez > 0) r += (uint32_t)ex * (uint32_t)ey * (uint32_t)ez;
+        }
+    }
+    return r;
+}
+
+// The cell tables of a handle, built once: ranks, bricks (an aligned block of
+// cells is one interval of ranks, and the bricks follow each other as the cells
+// of their own grid do), or, without bricks, each cell's neighbour ranks in
+// ascending order, no cell twice where an axis has fewer than three.
+__global__ void k_geometry(SimParams P, uint32_t *rank_of_cell, uint32_t *stencil, uint32_t *brick_lo, uint32_t *brick_hi,
+                           uint32_t *brick_ord)
+{
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < P.ncell; c += gridDim.x * blockDim.x) {
+        const int x = c % P.nc[0], y = c / P.nc[0] % P.nc[1], z = c / (P.nc[0] * P.nc[1]);
+        const uint32_t r = morton_rank(P.nc, x, y, z);
+        rank_of_cell[c] = r;
+        if (!P.use_bricks) {
+            uint32_t *st = stencil + (size_t)r * kStencil;
+            int m = 0;
+            for (int o = 0; o < kStencil; ++o) {
+                // offsets {-1, 0, 1}, {0, 1} or {0} along each axis
+                const int d[3] = {o % 3 - 1, o / 3 % 3 - 1, o / 9 - 1};
+                bool use = true;
+                for (int a = 0; a < 3; ++a)
+                    use = use && (P.nc[a] >= 3 || d[a] == 0 || (P.nc[a] == 2 && d[a] == 1));
+                if (!use) continue;
+                const uint32_t q = morton_rank(P.nc, (x + d[0] + P.nc[0]) % P.nc[0], (y + d[1] + P.nc[1]) % P.nc[1],
+                                               (z + d[2] + P.nc[2]) % P.nc[2]);
+                int k = m++;
+                for (; k > 0 && st[k - 1] > q; --k) st[k] = st[k - 1];
+                st[k] = q;
+            }
+            for (; m < kStencil; ++m) st[m] = kNone;
+        }
+    }
+    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < P.nbricks; b += gridDim.x * blockDim.x) {
+        const int x = b % P.nb[0], y = b / P.nb[0] % P.nb[1], z = b / (P.nb[0] * P.nb[1]);
+        const int ex = min(kBrick, P.nc[0] - x * kBrick), ey = min(kBrick, P.nc[1] - y * kBrick),
+                  ez = min(kBrick, P.nc[2] - z * kBrick);
+        const uint32_t lo = morton_rank(P.nc, x * kBrick, y * kBrick, z * kBrick);
+        brick_lo[b] = lo;
+        brick_hi[b] = lo + (uint32_t)(ex * ey * ez) - 1u;
+        brick_ord[b] = morton_rank(P.nb, x, y, z);
+    }
+}
+
 __global__ void k_bin(SimParams P, Ptrs D)
 {
     dependency_wait();
@@ -949,6 +1008,14 @@ __global__ void k_wait_probe(Ptrs D, uint32_t polls)
 cudaError_t launch_wait_probe(const Ptrs &D, uint32_t polls, cudaStream_t s)
 {
     k_wait_probe<<<1, 32, 0, s>>>(D, polls);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_geometry(const SimParams &P, const Ptrs &D, cudaStream_t s)
+{
+    k_geometry<<<grid_for(P.ncell), kThreads, 0, s>>>(P, (uint32_t *)D.rank_of_cell, (uint32_t *)D.stencil,
+                                                      (uint32_t *)D.brick_rank_lo, (uint32_t *)D.brick_rank_hi,
+                                                      (uint32_t *)D.brick_ord);
     return cudaGetLastError();
 }
 

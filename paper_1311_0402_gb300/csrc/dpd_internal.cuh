@@ -80,6 +80,8 @@ struct DevCtl {
     uint32_t rebuild_next;   // displacement flag raised by the kernel running now
     uint32_t done;           // blocks of the moving kernel that have finished (merged advance)
     uint32_t oparity;        // live set of the order arrays (tag, pid): flips only at a rebuild
+    uint32_t obs_done;       // blocks of the observables kernel that have finished
+    uint32_t pad0;
 };
 
 struct SimParams {
@@ -133,7 +135,7 @@ struct Ptrs {
                               // clears the other one for the next step
     float4 *fout;             // output of a standalone force evaluation
     DevCtl *ctl;
-    unsigned long long *obs;  // the 9 words of a dpd_obs, written by k_obs_finish
+    unsigned long long *obs;  // the 9 words of a dpd_obs, written by k_observe
     // cells
     const uint32_t *rank_of_cell;  // (cz * nc_y + cy) * nc_x + cx -> Morton rank
     const uint32_t *stencil;       // [ncell][27] neighbour ranks, ascending, kNone pad (without bricks)
@@ -214,10 +216,8 @@ cudaError_t launch_force(const SimParams &P, const Ptrs &D, int mode, bool out_f
 // kernels these launch: the opening phase 1 of a run, and the force phase of a step
 int phase1_kernels(const SimParams &P);
 int force_kernels(const SimParams &P);
-// observables: nblocks per-block partials in D.red, then their fixed-order
-// sum in D.red[nblocks * 8 .. + 8)
-cudaError_t launch_observe(const SimParams &P, const Ptrs &D, int nblocks, cudaStream_t s);
-cudaError_t launch_observe_finish(const Ptrs &D, int nblocks, int64_t n, double dof, double three_v, cudaStream_t s);
+// observables: the finished dpd_obs in D.obs (dof = 3N - 3 or 0, three_v = 3V)
+cudaError_t launch_observe(const SimParams &P, const Ptrs &D, double dof, double three_v, cudaStream_t s);
 // state transfer in the caller's layout (kernels_io.cu): validation of FP64
 // x, v and species (bits into *bad), conversion into the device layout, and
 // the scatter of a float4 array to FP64 triples in caller order

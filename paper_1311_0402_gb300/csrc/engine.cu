@@ -448,6 +448,13 @@ dpd_status guard(dpd_sim *h, bool need_state)
     return DPD_OK;
 }
 
+// Queue the observables of the live state: the finished record in D.obs.
+cudaError_t observe(dpd_sim *h)
+{
+    const double V = h->box[0] * h->box[1] * h->box[2];
+    return launch_observe(h->P, h->D, h->n > 1 ? 3.0 * h->n - 3.0 : 0.0, 3.0 * V, h->stream);
+}
+
 // Download a float4 array of the live order (c: the control words as read);
 // scatter xyz into out (n x 3).
 dpd_status download_xyz(dpd_sim *h, const DevCtl &c, const float4 *dev, double *out)
@@ -1035,11 +1042,8 @@ dpd_status dpd_observables(dpd_sim *h, dpd_obs *out)
     if (st) return st;
     if (!out) return fail(h, DPD_ERR_ARG, "out is NULL");
     // the record is finished on the device: one copy and one wait
-    const int nb = observe_blocks_for((int)h->n);
-    const double V = h->box[0] * h->box[1] * h->box[2];
     dpd_obs o;
-    CUDA_TRY(h, launch_observe(h->P, h->D, nb, h->stream));
-    CUDA_TRY(h, launch_observe_finish(h->D, nb, h->n, h->n > 1 ? 3.0 * h->n - 3.0 : 0.0, 3.0 * V, h->stream));
+    CUDA_TRY(h, observe(h));
     CUDA_TRY(h, cudaMemcpyAsync(&o, h->D.obs, sizeof(o), cudaMemcpyDeviceToHost, h->stream));
     st = wait(h);
     if (st) return st;
@@ -1051,7 +1055,7 @@ static_assert(sizeof(dpd_obs) == 9 * 8 && offsetof(dpd_obs, step) == 0 && offset
                   offsetof(dpd_obs, kinetic) == 16 && offsetof(dpd_obs, temperature) == 24 &&
                   offsetof(dpd_obs, virial) == 32 && offsetof(dpd_obs, pressure) == 40 &&
                   offsetof(dpd_obs, momentum) == 48,
-              "k_obs_finish writes dpd_obs as nine 8-byte words");
+              "k_observe writes dpd_obs as nine 8-byte words");
 
 dpd_status dpd_observables_async(dpd_sim *h, dpd_obs *out)
 {
@@ -1064,10 +1068,7 @@ dpd_status dpd_observables_async(dpd_sim *h, dpd_obs *out)
         cudaGetLastError();
         return fail(h, DPD_ERR_ARG, "out must be page-locked host memory");
     }
-    const int nb = observe_blocks_for((int)h->n);
-    const double V = h->box[0] * h->box[1] * h->box[2];
-    CUDA_TRY(h, launch_observe(h->P, h->D, nb, h->stream));
-    CUDA_TRY(h, launch_observe_finish(h->D, nb, h->n, h->n > 1 ? 3.0 * h->n - 3.0 : 0.0, 3.0 * V, h->stream));
+    CUDA_TRY(h, observe(h));
     CUDA_TRY(h, cudaMemcpyAsync(out, h->D.obs, sizeof(dpd_obs), cudaMemcpyDeviceToHost, h->stream));
     return DPD_OK;
 }

@@ -13,33 +13,6 @@ namespace {
 
 constexpr int kThreads = 256;
 
-// Deterministic block reduction of 8 doubles (fixed shuffle tree, then a
-// fixed order over the warps); thread 0 writes the block's partials.
-__device__ void block_reduce8(double (&v)[8], double *out)
-{
-    __shared__ double sh[8][kThreads / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        double x = v[k];
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xFFFFFFFFu, x, o);
-        if (lane == 0) sh[k][warp] = x;
-    }
-    __syncthreads();
-    if (threadIdx.x < 8) {
-        double s = 0.0;
-        for (int w = 0; w < kThreads / 32; ++w) s += sh[threadIdx.x][w];
-        out[threadIdx.x] = s;
-    }
-}
-
-// Observables, per-block partials of: sum v^2, sum v (3) over the
-// particles, and the virial sum over pairs inside r_c of r_ij . F^C_ij plus
-// the bonds' share (Eq. 3 and Sec. 4.5).  The virial comes from the force
-// evaluation that closed the last call (a force evaluation, or the last step
-// of a run): its positions are the current ones, and the pair kernel left one
-// partial per block in vir_part, summed here in a fixed order.  The kinetic
-// sums are exact to about 2^-48 per thread (Sum2), then FP64.
 // Error-free FP32 accumulation (FP64 arithmetic is scarce on this part):
 // s + c carries the exact running sum of a few dozen terms to about 2^-48
 // relative (Knuth's TwoSum for each addition; a square enters as its exact
@@ -62,36 +35,109 @@ struct Sum2 {
         c = __fadd_rn(c, fmaf(v, v, -hi));
     }
     __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+    // lane 0: the sum over the warp, in a fixed order
+    __device__ __forceinline__ void warp_reduce()
+    {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float s2 = __shfl_down_sync(0xFFFFFFFFu, s, o), c2 = __shfl_down_sync(0xFFFFFFFFu, c, o);
+            add(s2);
+            c = __fadd_rn(c, c2);
+        }
+    }
 };
 
-__global__ void __launch_bounds__(kThreads) k_observe(SimParams P, Ptrs D)
+// Observables: sum v^2, sum v (3) over the particles, and the virial sum over
+// pairs inside r_c of r_ij . F^C_ij plus the bonds' share (Eq. 3 and Sec. 4.5).
+// The virial comes from the force evaluation that closed the last call (a force
+// evaluation, or the last step of a run): its positions are the current ones,
+// and the pair kernel left one partial per block in vir_part, summed here in a
+// fixed order.  The kinetic sums are exact to about 2^-48 per warp (Sum2), then
+// FP64.  Each block leaves its partials in red; the last one to finish adds all of
+// them in block order (whichever it is, the order is the same) and stores the
+// finished dpd_obs, nine 8-byte words: step, n, kinetic, temperature, virial,
+// pressure, momentum[3], with the divisors 3N - 3 and 3V passed in.  One launch
+// and FP32 warp sums where three launches reduced in FP64: 81,000 particles, a
+// step and its record each time: 91 to 78 us a step.
+constexpr int kSums = 5;  // v^2, v (3), virial
+__global__ void __launch_bounds__(kThreads) k_observe(SimParams P, Ptrs D, double dof, double three_v)
 {
-    const float4 *__restrict__ vel = D.vel[D.ctl->parity];
-    Sum2 v2, px, py, pz;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < P.n; i += stride) {
+    __shared__ double sh[kSums][kThreads / 32];
+    __shared__ int s_last;
+    dependency_wait();
+    DevCtl *ctl = D.ctl;
+    const float4 *__restrict__ vel = D.vel[ctl->parity];
+    Sum2 sums[4];
+    double vir = 0.0;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x, first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    for (int64_t i = first; i < P.n; i += stride) {
         const float4 v = vel[i];
-        v2.add_square(v.x);
-        v2.add_square(v.y);
-        v2.add_square(v.z);
-        px.add(v.x);
-        py.add(v.y);
-        pz.add(v.z);
+        sums[0].add_square(v.x);
+        sums[0].add_square(v.y);
+        sums[0].add_square(v.z);
+        sums[1].add(v.x);
+        sums[2].add(v.y);
+        sums[3].add(v.z);
     }
-    double acc[8] = {v2.value(), px.value(), py.value(), pz.value(), 0, 0, 0, 0};
     const int64_t nvir = (P.ngroups + kForceWarps - 1) / kForceWarps;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nvir; k += stride) acc[4] += D.vir_part[k];
-    block_reduce8(acc, D.red + (size_t)blockIdx.x * 8);
-}
-
-// Sum of nb per-block partials (8 each) in a fixed order into out[0..7].
-__global__ void __launch_bounds__(kThreads) k_reduce8(const double *part, int nb, double *out)
-{
-    double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int b = threadIdx.x; b < nb; b += blockDim.x)
+    for (int64_t k = first; k < nvir; k += stride) vir += D.vir_part[k];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto warp_sum = [&](double x) {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) acc[k] += part[(size_t)b * 8 + k];
-    block_reduce8(acc, out);
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xFFFFFFFFu, x, o);
+        return x;
+    };
+    // the block's sum of sh[k] over the warps, on thread k
+    auto block_sums = [&]() {
+        __syncthreads();
+        double x = 0.0;
+        if (threadIdx.x < kSums)
+            for (int w = 0; w < kThreads / 32; ++w) x += sh[threadIdx.x][w];
+        __syncthreads();
+        return x;
+    };
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        sums[k].warp_reduce();
+        if (lane == 0) sh[k][warp] = sums[k].value();
+    }
+    // most warps hold no virial partial
+    if (__any_sync(0xFFFFFFFFu, first < nvir)) vir = warp_sum(vir);
+    if (lane == 0) sh[4][warp] = vir;
+    const double mine = block_sums();
+    if (threadIdx.x < kSums) {
+        D.red[(size_t)blockIdx.x * 8 + threadIdx.x] = mine;
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&ctl->obs_done, 1u) + 1u == gridDim.x;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (threadIdx.x == 0) ctl->obs_done = 0u;
+    double acc[kSums] = {0, 0, 0, 0, 0};
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += kThreads)
+#pragma unroll
+        for (int k = 0; k < kSums; ++k) acc[k] += __ldcg(D.red + (size_t)b * 8 + k);
+#pragma unroll
+    for (int k = 0; k < kSums; ++k) {
+        const double x = warp_sum(acc[k]);
+        if (lane == 0) sh[k][warp] = x;
+    }
+    const double total = block_sums();
+    if (threadIdx.x < kSums) sh[threadIdx.x][0] = total;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const double s0 = sh[0][0], virial = sh[4][0];
+        auto bits = [](double x) { return (unsigned long long)__double_as_longlong(x); };
+        D.obs[0] = ctl->step;
+        D.obs[1] = (unsigned long long)P.n;
+        D.obs[2] = bits(0.5 * s0);
+        D.obs[3] = bits(dof > 0.0 ? s0 / dof : 0.0);
+        D.obs[4] = bits(virial);
+        D.obs[5] = bits((s0 + virial) / three_v);
+        for (int k = 0; k < 3; ++k) D.obs[6 + k] = bits(sh[1 + k][0]);
+    }
 }
 
 __device__ __forceinline__ float axis_of(float4 x, int axis) { return axis == 0 ? x.x : (axis == 1 ? x.y : x.z); }
@@ -216,24 +262,6 @@ __global__ void k_pair_rng(uint64_t seed, uint32_t step, int64_t m, const uint32
     }
 }
 
-// One thread: the derived observables of the sums k_reduce8 left (v^2,
-// momentum, virial), by the same expressions as the host side of
-// dpd_observables with its divisors passed in (3N - 3 and 3V), stored as the
-// nine 8-byte words of a dpd_obs: step, n, kinetic, temperature, virial,
-// pressure, momentum[3].
-__global__ void k_obs_finish(const double *sums, const DevCtl *ctl, long long n, double dof, double three_v,
-                             unsigned long long *out)
-{
-    const double s0 = sums[0], vir = sums[4];
-    out[0] = ctl->step;
-    out[1] = (unsigned long long)n;
-    out[2] = (unsigned long long)__double_as_longlong(0.5 * s0);
-    out[3] = (unsigned long long)__double_as_longlong(dof > 0.0 ? s0 / dof : 0.0);
-    out[4] = (unsigned long long)__double_as_longlong(vir);
-    out[5] = (unsigned long long)__double_as_longlong((s0 + vir) / three_v);
-    for (int k = 0; k < 3; ++k) out[6 + k] = (unsigned long long)__double_as_longlong(sums[1 + k]);
-}
-
 }  // namespace
 
 int observe_blocks_for(int n)
@@ -242,17 +270,9 @@ int observe_blocks_for(int n)
     return g < 1 ? 1 : (g > 152 * 4 ? 152 * 4 : g);  // grid-stride beyond 4 blocks per SM
 }
 
-cudaError_t launch_observe(const SimParams &P, const Ptrs &D, int nblocks, cudaStream_t s)
+cudaError_t launch_observe(const SimParams &P, const Ptrs &D, double dof, double three_v, cudaStream_t s)
 {
-    k_observe<<<nblocks, kThreads, 0, s>>>(P, D);
-    k_reduce8<<<1, kThreads, 0, s>>>(D.red, nblocks, D.red + (size_t)nblocks * 8);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_observe_finish(const Ptrs &D, int nblocks, int64_t n, double dof, double three_v, cudaStream_t s)
-{
-    k_obs_finish<<<1, 1, 0, s>>>(D.red + (size_t)nblocks * 8, D.ctl, (long long)n, dof, three_v, D.obs);
-    return cudaGetLastError();
+    return launch_kernel(k_observe, observe_blocks_for(P.n), kThreads, 0, s, true, P, D, dof, three_v);
 }
 
 // Up to this many bins a block of one warp or more has its tables in the 48 KB

@@ -653,12 +653,9 @@ __device__ __forceinline__ void owner_pass_rows(const SimParams &P, const float4
     }
 }
 
-// One chunk against the owners [p_lo, p_hi) of cell slot t, kOwnersPerPass
-// owners at a time: every ballot of the pass over the NS live slots first
-// (no branches between them, so the tests overlap), then each owner's hits
-// are appended in turn, so an owner's entries stay contiguous in the list.
-constexpr int kOwnersPerPass = 1;
-
+// One chunk against the owners [p_lo, p_hi) of cell slot t, one at a time over
+// the NS live slots, so that an owner's entries stay contiguous in the list.
+//
 // ATOMIC (an ablation of the paper's Table 2, ballot against atomic
 // insertion): every hit takes its slot with an atomic add on the group's
 // shared counter instead of a ballot prefix; the list order then varies run
@@ -670,7 +667,6 @@ __device__ __forceinline__ uint32_t owner_pass(const SimParams &P, const float4 
                                                uint32_t c1, uint32_t first, uint32_t lane, uint32_t *list,
                                                uint32_t gcap, uint32_t total, uint32_t *count)
 {
-    constexpr int NO = kOwnersPerPass;
     const uint32_t lt = (1u << lane) - 1u;
     if constexpr (ATOMIC) {
         for (uint32_t p = p_lo; p < p_hi; ++p) {
@@ -690,33 +686,35 @@ __device__ __forceinline__ uint32_t owner_pass(const SimParams &P, const float4 
         }
         return total;
     } else {
-        for (uint32_t p = p_lo; p < p_hi; p += (uint32_t)NO) {
-            uint32_t m[NO][NS];
+        const float4 *own = s_pos + s_off[t];
+        for (uint32_t p = p_lo; p < p_hi; ++p) {
+            const uint32_t io = g_own + p;
+            const float4 pio = STAGED ? own[p] : pos[io];
+            // every ballot of the pass first (no branches between them, so the
+            // tests overlap); the hits stay in predicates for the stores.  The
+            // empty places of the last slot lie outside every cutoff.
+            bool hit[NS];
+            uint32_t m[NS], at = total;
 #pragma unroll
-            for (int o = 0; o < NO; ++o) {
-                const bool live = p + (uint32_t)o < p_hi;
-                const uint32_t po = live ? p + (uint32_t)o : p;
-                const uint32_t io = g_own + po;
-                const float4 pio = STAGED ? s_pos[s_off[t] + po] : pos[io];
-                const uint32_t k0 = HALF ? max(po + 1u, c0) : c0;
-#pragma unroll
-                for (int sl = 0; sl < NS; ++sl) {
-                    const uint32_t k = c0 + 32u * sl + lane;
-                    const uint32_t j = __float_as_uint(cand[sl].w);
-                    m[o][sl] = __ballot_sync(0xFFFFFFFFu, live & (k < c1) & (k >= k0) & within_list<WRAP>(P, cand[sl], pio) &
-                                                              (HALF || j != io));
-                }
+            for (int sl = 0; sl < NS; ++sl) {
+                hit[sl] = within_list<WRAP>(P, cand[sl], pio) &
+                          (HALF ? c0 + 32u * sl + lane > p : __float_as_uint(cand[sl].w) != io);
+                m[sl] = __ballot_sync(0xFFFFFFFFu, hit[sl]);
+                total += (uint32_t)__popc(m[sl]);
             }
-#pragma unroll
-            for (int o = 0; o < NO; ++o) {
-                const uint32_t entry_owner = (g_own + p + (uint32_t)o - first) << kOwnerShift;
+            const uint32_t entry_owner = (io - first) << kOwnerShift;
+            if (total <= gcap) {
 #pragma unroll
                 for (int sl = 0; sl < NS; ++sl) {
-                    if ((m[o][sl] >> lane) & 1u) {
-                        const uint32_t q = total + (uint32_t)__popc(m[o][sl] & lt);
-                        if (q < gcap) list[q] = entry_owner | __float_as_uint(cand[sl].w);
-                    }
-                    total += (uint32_t)__popc(m[o][sl]);
+                    if (hit[sl]) list[at + (uint32_t)__popc(m[sl] & lt)] = entry_owner | __float_as_uint(cand[sl].w);
+                    at += (uint32_t)__popc(m[sl]);
+                }
+            } else {  // counted, not written past the capacity
+#pragma unroll
+                for (int sl = 0; sl < NS; ++sl) {
+                    const uint32_t q = at + (uint32_t)__popc(m[sl] & lt);
+                    if (hit[sl] && q < gcap) list[q] = entry_owner | __float_as_uint(cand[sl].w);
+                    at += (uint32_t)__popc(m[sl]);
                 }
             }
         }
@@ -766,7 +764,7 @@ __device__ __forceinline__ uint32_t build_cell(const SimParams &P, const float4 
 #pragma unroll
         for (int sl = 0; sl < kSlots; ++sl) {
             const uint32_t kb = c0 + 32u * sl;
-            cand[sl] = make_float4(0.f, 0.f, 0.f, 0.f);
+            cand[sl] = make_float4(1.0e30f, 1.0e30f, 1.0e30f, 0.f);  // outside every cutoff
             if (kb < c1) {
                 // the cell of candidate kb + lane: the last cell starting at or
                 // below it in this slot, else the cell covering kb

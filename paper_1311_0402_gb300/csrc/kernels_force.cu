@@ -255,14 +255,13 @@ __device__ __forceinline__ bool force_epilogue(const SimParams &P, const Ptrs &D
 //   F = a_{t_i t_j} w - gamma w_R^2 (e . v_ij) + sigma/sqrt(dt) w_R xi_ij,
 //   f_i += F e_ij,  e_ij = (x_i - x_j) / r.
 // The 32 results of a batch are summed per owner by a segmented scan and
-// added to the owners' shared accumulators.  Deterministic mode (full lists,
-// each pair seen from both sides): the adds run in lane order, so every
-// force is summed in a fixed order.  Newton-3 mode (half lists): the adds
-// are shared-memory atomics, and the partner's share, -F e_ij, goes to
-// facc[j] by a global vector reduction.
+// added to the owners' shared accumulators.  Deterministic mode: full lists,
+// each pair seen from both sides, and every force is summed in a fixed order.
+// Newton-3 mode: half lists, and the partner's share, -F e_ij, goes to facc[j] by
+// a global vector reduction.
 // The epilogue adds bonds and the body force and, per MODE, writes the force
 // or integrates (see launch_force).
-constexpr int kQueue = 64;  // ring slots per warp (< 32 pending + 32 new)
+constexpr int kQueue = 128;  // ring slots per warp (< 32 pending + 64 new)
 
 // The candidate walk of a warp, templated on whether the minimum image can
 // be needed: a warp whose 32 particles all lie at least (r_list + skin) from
@@ -291,8 +290,18 @@ struct WarpSmem {
     float4 vi[32];
     float4 q[kQueue];      // (d, list entry: owner lane << kOwnerShift | j)
     uint8_t qo[kQueue];    // partner species (several species only)
-    float acc[3][32];
+    union {
+        float4 acc[32];            // plain adds (kPlainSums)
+        float acc3[3][32];         // atomics
+    };
 };
+
+// How a batch's run sums reach the owners' accumulators: by plain adds, or by
+// shared-memory atomics (us per launch, plain / atomics: 207,000 particles
+// deterministic 56 / 62, 786,000 amphiphile 92.1 / 94.2, 3,000,000 of one species
+// in Newton-3 mode 302.6 / 294.8).
+template <bool ONE_SPECIES, bool N3>
+constexpr bool kPlainSums = !(N3 && ONE_SPECIES);
 
 template <bool ONE_SPECIES, int SMODE, bool WRAP, bool N3, bool VIR>
 __device__ __forceinline__ void warp_pairs(const SimParams &P, const float4 *__restrict__ pos,
@@ -361,25 +370,34 @@ __device__ __forceinline__ void warp_pairs(const SimParams &P, const float4 *__r
             }
         }
         const bool tail_lane = owner < 32u && (lane == 31 || ((heads >> lane) & 2u) != 0u);
-        if (N3) {
+        if (!kPlainSums<ONE_SPECIES, N3>) {
             // an owner can recur in a later run of the batch: atomics
             if (tail_lane) {
-                atomicAdd(&w.acc[0][owner], sx);
-                atomicAdd(&w.acc[1][owner], sy);
-                atomicAdd(&w.acc[2][owner], sz);
+                atomicAdd(&w.acc3[0][owner], sx);
+                atomicAdd(&w.acc3[1][owner], sy);
+                atomicAdd(&w.acc3[2][owner], sz);
             }
         } else {
-            // fixed order: the runs add in lane order
+            // Fixed order.  The runs' owners are distinct unless the batch spans
+            // two chunks of a cell's candidates: then all add at once, otherwise
+            // in lane order.
+            auto add = [&]() {
+                float4 a = w.acc[owner];
+                a.x += sx;
+                a.y += sy;
+                a.z += sz;
+                w.acc[owner] = a;
+            };
             uint32_t tails = __ballot_sync(0xFFFFFFFFu, tail_lane);
-            while (tails) {
-                const int src = __ffs(tails) - 1;
-                if (lane == src) {
-                    w.acc[0][owner] += sx;
-                    w.acc[1][owner] += sy;
-                    w.acc[2][owner] += sz;
+            const uint32_t seen = __reduce_or_sync(0xFFFFFFFFu, tail_lane ? 1u << owner : 0u);
+            if (__popc(seen) == __popc(tails)) {
+                if (tail_lane) add();
+            } else {
+                while (tails) {
+                    if (lane == __ffs(tails) - 1) add();
+                    tails &= tails - 1u;
+                    __syncwarp();
                 }
-                tails &= tails - 1u;
-                __syncwarp();
             }
         }
         __syncwarp();
@@ -387,7 +405,7 @@ __device__ __forceinline__ void warp_pairs(const SimParams &P, const float4 *__r
 
     uint32_t head = 0u, tail = 0u;
     // one candidate (entry e, partner position pj): test it, queue it if
-    // inside r_c, evaluate a full batch
+    // inside r_c
     auto candidate = [&](bool act, uint32_t e, float4 pj) {
         const uint32_t own = e >> kOwnerShift;
         if (kChecked && act && ((e & kIndexMask) >= (uint32_t)P.n || own >= owners)) {
@@ -406,40 +424,37 @@ __device__ __forceinline__ void warp_pairs(const SimParams &P, const float4 *__r
             if (!ONE_SPECIES) w.qo[slot] = (uint8_t)((uint32_t)__float_as_int(pj.w));
         }
         tail += (uint32_t)__popc(m);
-        __syncwarp();
-        if (tail - head >= 32u) {
-            run_batch(head, 32);
-            head += 32u;
-        }
     };
-    // Entries are loaded four iterations ahead through a register rotation
-    // (the loop stays rolled: the batch evaluation inside it is large), and
-    // each candidate's position one ahead.  Past the end a lane reads entry 0
-    // (owner 0, particle 0), a valid address that the act flag discards.
     auto entry = [&](uint32_t k) -> uint32_t { return k < nent ? __ldg(list + k) : 0u; };
-    // (the checked build clamps the prefetch index into range; the candidate
-    // test then rejects the entry)
     auto at = [&](uint32_t e) -> uint32_t {
         const uint32_t j = e & kIndexMask;
         return (kChecked && j >= (uint32_t)P.n) ? 0u : j;
     };
     const uint32_t l = (uint32_t)lane;
-    uint32_t e0 = entry(l), e1 = entry(32u + l), e2 = entry(64u + l), e3 = entry(96u + l);
-    float4 pc = __ldg(pos + at(e0));
-    for (uint32_t base = 0; base < nent; base += 32u) {
-        const uint32_t e4 = entry(base + 128u + l);
-        const float4 pn = __ldg(pos + at(e1));
-        candidate(base + l < nent, e0, pc);
-        e0 = e1;
-        e1 = e2;
-        e2 = e3;
-        e3 = e4;
-        pc = pn;
-    }
-    while (tail != head) {
-        const int nb = (int)min(32u, tail - head);
-        run_batch(head, nb);
-        head += (uint32_t)nb;
+    // Two entries a lane and iteration: their positions are fetched together and
+    // the tests overlap, with the batch evaluation, which is large, in the code
+    // once.  294.8 us per launch on the 3M fluid; one entry an iteration with its
+    // position fetched one ahead 312, three entries 307, two with positions one
+    // ahead (48 registers, 10 blocks) 304.8.
+    uint32_t e0 = entry(l), e1 = entry(32u + l);
+    for (uint32_t base = 0;; base += 64u) {
+        const bool more = base < nent;
+        if (more) {
+            const float4 p0 = __ldg(pos + at(e0)), p1 = __ldg(pos + at(e1));
+            const uint32_t e2 = entry(base + 64u + l), e3 = entry(base + 96u + l);
+            candidate(base + l < nent, e0, p0);
+            candidate(base + 32u + l < nent, e1, p1);
+            e0 = e2;
+            e1 = e3;
+            __syncwarp();
+        }
+        const uint32_t need = more ? 32u : 1u;
+        while (tail - head >= need) {
+            const int nb = (int)min(32u, tail - head);
+            run_batch(head, nb);
+            head += (uint32_t)nb;
+        }
+        if (!more) break;
     }
 }
 
@@ -464,7 +479,7 @@ __device__ __forceinline__ void block_sum_double(float x, double *out)
 // whose positions are the state the observables describe.
 // 12 resident blocks per SM (48 warps) caps the kernel at 40 registers: the
 // walk's scattered gathers need the extra warps to hide their latency
-// (measured on the 3M fluid: 0.311 ms per launch against 0.338 ms at the
+// (measured on the 3M fluid, an earlier walk: 0.311 ms per launch against 0.338 ms at the
 // compiler's 47 registers and 10 blocks; 32 registers spill and take 0.474).
 constexpr int kForceMinBlocks = 12;
 template <bool ONE_SPECIES, int SMODE, int MODE, bool LHALF, bool N3, bool VIR>
@@ -495,9 +510,7 @@ __global__ void __launch_bounds__(kForceThreads, kForceMinBlocks) k_force(SimPar
     const float4 vi = valid ? vel[i] : make_float4(0.f, 0.f, 0.f, 0.f);
     w.pi[lane] = pi;
     w.vi[lane] = vi;
-    w.acc[0][lane] = 0.f;
-    w.acc[1][lane] = 0.f;
-    w.acc[2][lane] = 0.f;
+    w.acc[lane] = make_float4(0.f, 0.f, 0.f, 0.f);  // (as long as the whole of acc3)
     // the warp may skip the minimum image when all its particles are far from the faces
     const bool interior = !valid || (pi.x >= P.wrap_margin && pi.x <= P.L[0] - P.wrap_margin &&
                                      pi.y >= P.wrap_margin && pi.y <= P.L[1] - P.wrap_margin &&
@@ -516,7 +529,9 @@ __global__ void __launch_bounds__(kForceThreads, kForceMinBlocks) k_force(SimPar
     else
         warp_pairs<ONE_SPECIES, SMODE, true, N3, VIR>(P, pos, vel, list, nent, lane, w, a_tab, facc, vir, owners, bad);
     if (kChecked && __any_sync(0xFFFFFFFFu, bad) && lane == 0) atomicOr(&ctl->err, kErrBadIndex);
-    float fx = w.acc[0][lane], fy = w.acc[1][lane], fz = w.acc[2][lane];
+    constexpr bool plain = kPlainSums<ONE_SPECIES, N3>;
+    float fx = plain ? w.acc[lane].x : w.acc3[0][lane], fy = plain ? w.acc[lane].y : w.acc3[1][lane],
+          fz = plain ? w.acc[lane].z : w.acc3[2][lane];
 
     if (N3) {
         // this group's share of particle i's force joins the shares other

@@ -78,7 +78,7 @@ struct DevCtl {
     unsigned long long nrebuild;
     uint32_t max_nnb;        // largest group list total (pair entries) of the last build
     uint32_t rebuild_next;   // displacement flag raised by the kernel running now
-    uint32_t done;           // blocks of the moving kernel that have finished (merged advance)
+    uint32_t done;           // blocks of the running kernel that have finished (merged advance, small sort)
     uint32_t oparity;        // live set of the order arrays (tag, pid): flips only at a rebuild
     uint32_t obs_done;       // blocks of the observables kernel that have finished
     uint32_t pad0;
@@ -118,7 +118,7 @@ struct SimParams {
     int no_reorder;           // 1: particles stay in load order (ablation; tile builder, no bricks)
     int list_layout;          // 0: packed group lists; 1: rows per particle (double insertion, join,
                               // 32x32 tile transpose; full lists, one thread per particle in the force)
-    int sort_small;           // the rebuild's sort runs in one block
+    int sort_small;           // the rebuild's sort is one launch
     int group;                // particles per group list: 32, 16, 8 or 4
     int brick_split;          // CTAs of the builder per brick
     int brick_cap;            // halo particles the brick builder stages in shared memory
@@ -240,7 +240,7 @@ cudaError_t launch_pair_rng(uint64_t seed, uint64_t step, int64_t m, const uint3
 // the tables D.rank_of_cell, D.brick_* or D.stencil, once per handle
 cudaError_t launch_geometry(const SimParams &P, const Ptrs &D, cudaStream_t s);
 int scan_blocks_for(int ncell);
-// whether a box's binning, scan and reorder fit one block (k_sort_small), and
+// whether a box's binning, scan and reorder fit a block's shared memory (k_sort_small), and
 // the kernels of a rebuild
 bool sort_fits_block(int64_t n, int ncell);
 int rebuild_kernels(const SimParams &P, int n_scan_blocks);

@@ -301,8 +301,8 @@ dpd_status dpd_get_state(dpd_sim *h, double *x, double *v, uint64_t *step);
 
 /* Number of particles, of neighbour-list rebuilds so far (the rebuild branch
  * of Algorithm 1) and the list capacity per particle; each output nullable.
- * Waits for the queued work; without a state n, rebuilds and the capacity
- * read 0. */
+ * Waits for the queued work if rebuilds is asked for (the others are known on
+ * the host); without a state n, rebuilds and the capacity read 0. */
 dpd_status dpd_info(dpd_sim *h, int64_t *n, int64_t *rebuilds, int32_t *nbr_capacity);
 
 /* Issue-rate probe for the denominator of the ALU roofline the pair kernel

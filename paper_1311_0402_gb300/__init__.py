@@ -303,7 +303,6 @@ def dpd_set_state(h, x, v, species=None, tag=None, step=0):
     tg = None if tag is None else np.ascontiguousarray(tag, np.uint32)
     _check(lib().dpd_set_state(h, x.shape[0], _p(x, ctypes.c_double), _p(v, ctypes.c_double),
                                _p(sp, ctypes.c_int32), _p(tg, ctypes.c_uint32), step), h)
-    h.n = x.shape[0]  # the size of the arrays read back
 
 
 def dpd_set_bonds(h, pairs, k, r0):
@@ -330,10 +329,9 @@ def dpd_info(h):
 
 
 def _nvec(h):
-    # the last load's count (dpd_info would wait for the queued work first);
-    # None for a handle loaded elsewhere
-    n = getattr(h, "n", None)
-    return dpd_info(h)["n"] if n is None else n
+    n = ctypes.c_int64()
+    _check(lib().dpd_info(h, ctypes.byref(n), None, None), h)  # (without the rebuilds: no wait)
+    return n.value
 
 
 def dpd_forces(h) -> np.ndarray:

@@ -1131,7 +1131,7 @@ dpd_status dpd_info(dpd_sim *h, int64_t *n, int64_t *rebuilds, int32_t *nbr_capa
     if (st) return st;
     DevCtl c;
     std::memset(&c, 0, sizeof(c));
-    if (h->has_state) {
+    if (h->has_state && rebuilds) {  // only the device counts them
         st = read_ctl(h, c);
         if (st) return st;
     }

@@ -75,8 +75,7 @@ def parse():
                     help="also time the atomic-insertion list builder against the ballot one (Table 2), "
                          "reorder on/off and the paper's row list layout against the packed lists")
     ap.add_argument("--no-conditional", action="store_true",
-                    help="launch the rebuild chain in every step's graph (for profilers that do not enter "
-                         "conditional graph nodes)")
+                    help="no effect: the rebuild chain is launched in every step's graph")
     return ap.parse_args()
 
 

@@ -143,6 +143,18 @@ size_t footprint(int64_t n, int ncell, bool lhalf, int threads)
     return ens_layout((int)n, ncell, lhalf, threads).total;
 }
 
+// The shared memory a box is accepted by: 53 B a particle (69 with vh), 8 B a
+// cell and 6 KB.  It is at least the footprint of a launch of kMinThreads
+// threads, so an accepted box always has a launch shape.
+constexpr int kMinThreads = 64;
+static_assert(kMinThreads / 32 * kEnsWarpBytes <= 6144, "a box that is accepted must have a launch shape");
+
+size_t accepted_bytes(int64_t n, int ncell, bool lhalf)
+{
+    const EnsLayout l = ens_layout((int)n, ncell, lhalf, 0);
+    return l.total + ens_align16((size_t)n * 2) + 6144;
+}
+
 // Size class: how many CTAs of the box's footprint (256 threads) fit on one
 // SM -- 1 (class 0), 2, 3, or 4 and more (class 3).
 int class_of(int64_t n, int ncell, bool lhalf, size_t limit)
@@ -293,7 +305,7 @@ bool shape_for(const std::vector<const EBox *> &bs, bool lhalf, int s_mode, bool
 bool pick_shape(const std::vector<const EBox *> &bs, bool lhalf, int s_mode, bool n3, int threads, int cluster,
                 size_t limit, Shape &out)
 {
-    for (int t = threads; t >= 128; t /= 2)
+    for (int t = threads; t >= kMinThreads; t /= 2)
         for (int c = cluster; c >= 1; c /= 2)
             if (shape_for(bs, lhalf, s_mode, n3, t, c, limit, out)) return true;
     return false;
@@ -370,7 +382,7 @@ int32_t dpd_ensemble_fits(const dpd_box_params *p, int64_t n)
     if (!check_params(p, n, nc).empty()) return 0;
     const size_t limit = ensemble_smem_limit();
     if (limit == 0) return 0;
-    return footprint(n, nc[0] * nc[1] * nc[2], p->lambda == 0.5, 128) <= limit ? 1 : 0;
+    return accepted_bytes(n, nc[0] * nc[1] * nc[2], p->lambda == 0.5) <= limit ? 1 : 0;
 }
 
 dpd_status dpd_ensemble_add(dpd_ensemble *e, const dpd_box_params *p, int64_t n, const double *x, const double *v,
@@ -383,7 +395,7 @@ dpd_status dpd_ensemble_add(dpd_ensemble *e, const dpd_box_params *p, int64_t n,
     if (!why.empty()) return efail(e, DPD_ERR_ARG, why);
     const int ncell = nc[0] * nc[1] * nc[2];
     const bool lhalf = p->lambda == 0.5;
-    if (footprint(n, ncell, lhalf, 128) > e->limit)
+    if (accepted_bytes(n, ncell, lhalf) > e->limit)
         return efail(e, DPD_ERR_ARG, "box does not fit one CTA's shared memory (" + std::to_string(n) + " particles)");
 
     EBox b;

@@ -147,3 +147,22 @@ def test_ensemble_forces_of_sparse_and_dense_boxes(n, L, lam, shape):
     e.sync()
     assert np.isfinite(e.state(i)[0]).all()
     e.close()
+
+
+def test_ensemble_runs_a_sparse_box_at_the_limit():
+    """A box of few particles and many cells, the largest that is accepted,
+    has a launch shape."""
+    need_gpu()
+    n, fits = 60, 0.0
+    L = 25.0
+    while dpd.dpd_ensemble_fits((L, 30.0, 30.0), [[25.0]], 4.5, 1.0, 1.0, 1.0, 0.01, n):
+        fits, L = L, L + 1.01
+    assert fits > 0.0
+    box = (fits, 30.0, 30.0)
+    x, v = workloads.uniform_fluid(box, n, 1.0, 3)[:2]
+    e = dpd.Ensemble()
+    i = e.add(box, [[25.0]], 4.5, 1.0, 1.0, 1.0, 0.01, x, v)
+    e.step(2)
+    e.sync()
+    assert e.state(i)[2] == 2
+    e.close()

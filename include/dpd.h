@@ -64,7 +64,7 @@ typedef struct {
     double lambda;            /* velocity-Verlet prediction factor (default 0.5) */
     double body_force[3];     /* g (force per particle, unit mass) */
     int32_t nbr_capacity;     /* list capacity per particle: particles are listed in
-                                 groups of 32 consecutive ones, each group holding
+                                 groups of up to 32 consecutive ones, each group holding
                                  up to 32 x nbr_capacity pair entries; 0 = from the
                                  density, grown when a build overflows */
     int32_t graph_steps;      /* steps per captured CUDA graph (default 8; 0 = no graphs) */
@@ -88,7 +88,7 @@ typedef struct {
                                  into cell order (Sec. 3.2); 1: they stay in load order and
                                  the list is built through the sort permutation -- the
                                  paper's reorder on/off comparison (Sec. 3.2); slower */
-    int32_t list_layout;      /* 0 (default): packed lists per group of 32 particles (see
+    int32_t list_layout;      /* 0 (default): packed lists per group of particles (see
                                  nbr_capacity), consumed 32 entries at a time; 1: the
                                  paper's layout (Sec. 3.3): one row of nbr_capacity entries
                                  per particle, written row-major by the builder with the

@@ -104,7 +104,9 @@ dpd_status dpd_server_create(const dpd_server_options *o, dpd_server **out);
 
 /* Queue a box; *ticket identifies it.  The request is validated here
  * (DPD_ERR_ARG, nothing queued) and its arrays copied.  A box whose
- * estimated memory exceeds the whole budget is refused with DPD_ERR_OOM. */
+ * estimated memory exceeds the whole budget is refused with DPD_ERR_OOM; the
+ * estimate is of lists of 32 particles a group, and a box whose smaller groups
+ * take more counts with those, at most as the whole budget. */
 dpd_status dpd_server_submit(dpd_server *s, const dpd_request *r, uint64_t *ticket);
 
 /* Wait up to timeout_s seconds for a box to finish; fills *res and, when

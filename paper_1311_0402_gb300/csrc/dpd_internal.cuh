@@ -12,9 +12,9 @@
 //   force[p] float4 (fx, fy, fz, 0)                       16 B
 //   tag[p]   u32 identity tag (keys the random force)
 //   pid[p]   u32 caller's particle index
-// Neighbour list, packed per group: a group is a run of at most 32
-// consecutive particles (the particles of one brick in 32s, or 32-aligned
-// tiles when there are no bricks).  Group g's pairs are one dense run of
+// Neighbour list, packed per group: a group is a run of at most P.group (4 to
+// 32) consecutive particles (the particles of one brick in runs of P.group, or
+// 32-aligned tiles when there are no bricks).  Group g's pairs are one dense run of
 // 32-bit entries at nbr[g * gcap], entry = (owner lane << 27) | j for the
 // pair of particle first + lane with particle j; gdesc[g] = (first,
 // owners | entries << 6).  A warp reads 32 consecutive entries in one
@@ -43,6 +43,7 @@ constexpr int64_t kMaxParticles = int64_t(1) << kOwnerShift;
 constexpr int kGroup = 32;                            // particles per group (one warp)
 constexpr int kMinGroup = 4;
 constexpr int kGroupsWanted = 10000;
+constexpr double kSmallGroupBytes = 1024.0 * 1024 * 1024;  // what the lists of groups below 32 may take
 constexpr int kBuildWarps = 8;                        // warps per block of the brick builder
 constexpr int kBuildBlocksWanted = 1024;
 constexpr int kForceWarps = 4;                        // groups per block of the pair kernel
@@ -89,7 +90,7 @@ struct SimParams {
     int ncell;
     int nc[3];
     int cap;                  // neighbour capacity per particle (a group holds 32 x cap entries)
-    int gcap;                 // entries per group list = group * cap
+    int gcap;                 // entries per group list = 32 * cap, whatever the group
     int ngroups;              // group descriptors (lists) in use
     float L[3];
     float halfL[3];
@@ -164,6 +165,26 @@ struct Ptrs {
 };
 
 // ----------------------------------------------------------------- helpers
+// Bytes of the lists of n particles in groups of `group` over nbricks bricks.
+// A list of any group holds 32 cap entries: those of a smaller group are among
+// those of the 32 particles it belongs to, so whatever spot condenses in a run
+// fits it if it fits a list of 32.
+inline double group_list_bytes(int64_t n, double nbricks, double cap, int group)
+{
+    return ((double)n / group + nbricks) * kGroup * cap * 4.0;
+}
+
+// Particles per group list of a box with bricks, of which `handles` run side by
+// side (the rule and its figures: pick_groups in engine.cu).
+inline int group_for(int64_t n, double nbricks, double cap, int handles)
+{
+    int group = kGroup;
+    while (group > kMinGroup && n < (int64_t)(kGroupsWanted / handles) * group &&
+           group_list_bytes(n, nbricks, cap, group / 2) <= kSmallGroupBytes)
+        group /= 2;
+    return group;
+}
+
 __host__ __device__ inline uint32_t ceil_div_u(uint32_t a, uint32_t b) { return (a + b - 1) / b; }
 
 // Kernels of a step follow each other by programmatic dependent launch: each

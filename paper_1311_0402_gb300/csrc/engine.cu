@@ -312,8 +312,8 @@ dpd_status get_graph(dpd_sim *h, int k, cudaGraphExec_t *out)
     return DPD_OK;
 }
 
-// Group lists: with bricks, brick b's groups take ids from lo_b / 32 +
-// ord(b), so n / 32 + nbricks ids cover every brick; otherwise 32-aligned
+// Group lists: with bricks, brick b's groups take ids from lo_b / group +
+// ord(b), so n / group + nbricks ids cover every brick; otherwise 32-aligned
 // tiles.
 int group_count(const dpd_sim *h, int64_t n)
 {
@@ -330,28 +330,36 @@ int group_count(const dpd_sim *h, int64_t n)
 // 3,000 particles 46.6 / - / 26.8 / 24.0; 32,000 (rho = 4) 61.9 / 44.0 / 33.8 /
 // 33.5; 81,000 56.7 / 44.6 / 43.2 / 45.7; 207,000 73.5 / 68.4 / 69.6 / -;
 // 648,000 155.3 / 156.0 / - / -; 3,000,000 575 / 604 / - / -, and a split of
-// 2 there 591.  A fixed capacity keeps groups of 32, whose particles share it.
-// Handles that run side by side each want their share of the chip only (in
-// deterministic mode the groups, which order the sums, stay those of a handle
-// alone).
-void pick_groups(dpd_sim *h, int64_t n)
+// 2 there 591.  A fixed capacity keeps groups of 32, whose particles share it;
+// so do lists that would take more than kSmallGroupBytes (a box of thousands of
+// particles at hundreds of neighbours each).  Handles that run side by side each
+// want their share of the chip only (in deterministic mode the groups, which
+// order the sums, stay those of a handle alone).
+void set_group(dpd_sim *h, int64_t n, int group)
 {
     SimParams &P = h->P;
-    P.group = kGroup;
+    P.group = group;
     P.brick_split = 1;
     if (!P.use_bricks) return;
-    if (P.list_layout == 0 && h->opt.nbr_capacity == 0)
-        while (P.group > kMinGroup && n < (int64_t)(kGroupsWanted / (h->P.newton3 ? h->share : 1)) * P.group) P.group /= 2;
     const int64_t rounds = (n / P.nbricks + P.group * kBuildWarps - 1) / (P.group * kBuildWarps);
     P.brick_split = (int)std::max<int64_t>(1, std::min<int64_t>(kBuildBlocksWanted / h->share / P.nbricks, rounds));
 }
 
-// per-particle capacity from the largest group total of a build
-int capacity_for_total(uint32_t max_total, int group)
+void pick_groups(dpd_sim *h, int64_t n, int cap)
 {
-    int cap = (int)(((uint64_t)max_total * 5 / 4 + 64 + group - 1) / group);
+    const SimParams &P = h->P;
+    const bool any = P.use_bricks && P.list_layout == 0 && h->opt.nbr_capacity == 0;
+    set_group(h, n, any ? group_for(n, P.nbricks, cap, P.newton3 ? h->share : 1) : kGroup);
+}
+
+// per-particle capacity from the largest total of a build's groups of 32
+int capacity_for_total(uint32_t max_total)
+{
+    int cap = (int)(((uint64_t)max_total * 5 / 4 + 64 + kGroup - 1) / kGroup);
     return std::max((cap + 7) / 8 * 8, 32);
 }
+
+size_t list_bytes(const dpd_sim *h, int cap) { return (size_t)h->P.ngroups * kGroup * (size_t)cap * sizeof(uint32_t); }
 
 int auto_capacity(const dpd_sim *h, int64_t n)
 {
@@ -392,7 +400,7 @@ dpd_status alloc_particles(dpd_sim *h, int64_t n, int cap)
     h->P.ngroups = group_count(h, n);
     A((void **)&D.gdesc, sizeof(uint2) * (size_t)h->P.ngroups);
     A((void **)&D.rowcnt, u4);
-    A((void **)&D.nbr, (size_t)h->P.ngroups * h->P.group * (size_t)cap * sizeof(uint32_t));
+    A((void **)&D.nbr, list_bytes(h, cap));
     h->red_doubles = std::max<size_t>((size_t)observe_blocks_for((int)n) * 8 + 8, 4096);
     A((void **)&D.vir_part, sizeof(double) * (size_t)((h->P.ngroups + kForceWarps - 1) / kForceWarps));
     A((void **)&D.red, h->red_doubles * sizeof(double));
@@ -406,8 +414,24 @@ dpd_status alloc_particles(dpd_sim *h, int64_t n, int cap)
                                 h->stream));
     for (int b = 0; b < 2; ++b) CUDA_TRY(h, cudaMemsetAsync(D.facc[b], 0, f4, h->stream));
     h->P.cap = cap;
-    h->P.gcap = h->P.group * cap;
+    h->P.gcap = kGroup * cap;
     h->cap_alloc_n = n;
+    return DPD_OK;
+}
+
+// The lists anew, in groups of `group` and of capacity cap (the particle arrays
+// stay); without memory for them there are none.
+dpd_status relist(dpd_sim *h, int group, int cap)
+{
+    if (h->D.nbr) dev_free(h, h->D.nbr, h->allocs);
+    h->D.nbr = nullptr;
+    set_group(h, h->n, group);
+    h->P.ngroups = group_count(h, h->n);
+    drop_graphs(h);
+    dpd_status st = dev_alloc(h, (void **)&h->D.nbr, list_bytes(h, cap), h->allocs);
+    if (st) return st;
+    h->P.cap = cap;
+    h->P.gcap = kGroup * cap;
     return DPD_OK;
 }
 
@@ -422,20 +446,33 @@ dpd_status rebuild_and_force(dpd_sim *h, bool grow_on_overflow)
         CUDA_TRY(h, launch_force(h->P, h->D, kForceEval, false, h->stream, true));
         DevCtl c;
         dpd_status st = check_err(h, c);
-        if (st != DPD_ERR_NBR_OVERFLOW || !grow_on_overflow) return st;
-        // grow the list: keep the particle arrays, reallocate the table (the
-        // row layout reports its longest row, the packed one its largest group)
-        const int cap = h->P.list_layout == 1 ? ((int)((uint64_t)c.max_nnb * 5 / 4 + 8) + 31) / 32 * 32
-                                              : capacity_for_total(c.max_nnb, h->P.group);
-        if ((int64_t)cap * h->P.group >= (int64_t(1) << 26))
-            return fail(h, DPD_ERR_NBR_OVERFLOW, "neighbour list overflow: group list beyond 2^26 entries");
-        dev_free(h, h->D.nbr, h->allocs);
-        st = dev_alloc(h, (void **)&h->D.nbr, (size_t)h->P.ngroups * h->P.group * (size_t)cap * sizeof(uint32_t),
-                       h->allocs);
-        if (st) return st;
-        h->P.cap = cap;
-        h->P.gcap = h->P.group * cap;
-        drop_graphs(h);
+        const int group = h->P.group;
+        const bool uneven = st == DPD_OK && group < kGroup && c.max_nnb > (uint32_t)(group * h->P.cap);
+        if (!grow_on_overflow || (st != DPD_ERR_NBR_OVERFLOW && !uneven)) return st;
+        if (group < kGroup) {
+            // 32 particles may need up to 32 / group times the largest list: a
+            // capacity from that bound leaves a run the room that lists of 32
+            // grown to their largest total would; where it takes too much
+            // memory, groups of 32, whose build tells what they need
+            const uint64_t bound = (uint64_t)c.max_nnb * (kGroup / group);
+            const int cap = bound < (uint64_t(1) << 25) ? capacity_for_total((uint32_t)bound) : 0;
+            const bool keep = cap > 0 && group_list_bytes(h->n, h->P.nbricks, cap, group) <= kSmallGroupBytes;
+            st = keep ? relist(h, group, cap) : DPD_ERR_OOM;
+            if (st) st = relist(h, kGroup, h->P.cap);
+        } else {
+            // grow the list (the row layout reports its longest row, the packed
+            // one its largest group)
+            const int cap = h->P.list_layout == 1 ? ((int)((uint64_t)c.max_nnb * 5 / 4 + 8) + 31) / 32 * 32
+                                                  : capacity_for_total(c.max_nnb);
+            if ((int64_t)cap * kGroup >= (int64_t(1) << 26))
+                return fail(h, DPD_ERR_NBR_OVERFLOW, "neighbour list overflow: group list beyond 2^26 entries");
+            st = relist(h, group, cap);
+        }
+        if (st) {  // no lists: the next state allocates all
+            h->has_state = false;
+            h->cap_alloc_n = -1;
+            return st;
+        }
     }
     return fail(h, DPD_ERR_NBR_OVERFLOW, "neighbour list overflow after regrowing");
 }
@@ -699,11 +736,15 @@ dpd_status dpd_set_state(dpd_sim *h, int64_t n, const double *x, const double *v
         h->P.brick_cap = std::min(std::max(bc, 256), std::min(max_brick_cap(), 65535));
     }
     h->P.sort_small = sort_fits_block(n, h->P.ncell) ? 1 : 0;
-    pick_groups(h, n);
-    if (n != h->n || cap != h->P.cap || h->cap_alloc_n != n) {
+    pick_groups(h, n, cap);
+    if (n != h->n || cap != h->P.cap || h->cap_alloc_n != n || group_count(h, n) != h->P.ngroups) {
         h->n = n;
         h->P.n = (int)n;
         st = alloc_particles(h, n, cap);
+        if (st == DPD_ERR_OOM && h->P.group < kGroup) {  // the lists of 32 take less
+            set_group(h, n, kGroup);
+            st = alloc_particles(h, n, cap);
+        }
         if (st) {
             h->has_state = false;
             return st;
@@ -779,9 +820,13 @@ dpd_status dpd_get_neighbors(dpd_sim *h, int64_t cap, uint32_t *pairs_out, int64
     if (st) return st;
     const int64_t n = h->n;
     int G = h->P.ngroups;
-    std::vector<uint32_t> nbr((size_t)G * h->P.gcap), pid(n);
+    // of each packed list as much as the longest one holds; the rows whole
+    const size_t gcap = (size_t)h->P.gcap;
+    const size_t width = h->P.list_layout == 1 ? gcap : std::min<size_t>(gcap, std::max<uint32_t>(c.max_nnb, 1u));
+    std::vector<uint32_t> nbr((size_t)G * width), pid(n);
     std::vector<uint2> desc(G);
-    CUDA_TRY(h, cudaMemcpyAsync(nbr.data(), h->D.nbr, sizeof(uint32_t) * nbr.size(), cudaMemcpyDeviceToHost, h->stream));
+    CUDA_TRY(h, cudaMemcpy2DAsync(nbr.data(), width * sizeof(uint32_t), h->D.nbr, gcap * sizeof(uint32_t),
+                                  width * sizeof(uint32_t), (size_t)G, cudaMemcpyDeviceToHost, h->stream));
     CUDA_TRY(h, cudaMemcpyAsync(desc.data(), h->D.gdesc, sizeof(uint2) * G, cudaMemcpyDeviceToHost, h->stream));
     CUDA_TRY(h, cudaMemcpyAsync(pid.data(), h->D.pid[c.oparity], sizeof(uint32_t) * n, cudaMemcpyDeviceToHost, h->stream));
     st = wait(h);
@@ -809,9 +854,9 @@ dpd_status dpd_get_neighbors(dpd_sim *h, int64_t cap, uint32_t *pairs_out, int64
     }
     for (int g = 0; g < G; ++g) {
         const uint32_t first = desc[g].x, owners = desc[g].y & 63u, ne = desc[g].y >> 6;
-        if (owners > (uint32_t)kGroup || ne > (uint32_t)h->P.gcap || (owners && first + owners > (uint64_t)n))
+        if (owners > (uint32_t)kGroup || ne > width || (owners && first + owners > (uint64_t)n))
             return fail(h, DPD_ERR_STATE, "corrupt group descriptor");
-        const uint32_t *list = nbr.data() + (size_t)g * h->P.gcap;
+        const uint32_t *list = nbr.data() + (size_t)g * width;
         for (uint32_t k = 0; k < ne; ++k) {
             const uint32_t own = list[k] >> kOwnerShift, j = list[k] & kIndexMask;
             if (own >= owners || j >= (uint32_t)n) return fail(h, DPD_ERR_STATE, "neighbour entry out of range");

@@ -65,9 +65,9 @@ struct Slot {
 
 // Device bytes of one box, following the engine's allocations: the
 // double-buffered particle arrays and scratch (about 300 B per particle), the
-// list at the automatic capacity (32 entries per particle group slot), the
-// cell tables, and a fixed allowance.
-double estimate_bytes(const Job &j, const dpd_options &o)
+// lists at the automatic capacity (of groups as small as the engine may choose,
+// or, small = false, of 32 particles), the cell tables, and a fixed allowance.
+double estimate_bytes(const Job &j, const dpd_options &o, bool small)
 {
     const double V = j.box[0] * j.box[1] * j.box[2];
     const double rl = j.rc + (j.skin > 0.0 ? j.skin : o.skin);
@@ -76,8 +76,9 @@ double estimate_bytes(const Job &j, const dpd_options &o)
     cap = std::ceil(cap / 8.0) * 8.0;
     double ncell = 1.0;
     for (int a = 0; a < 3; ++a) ncell *= std::max(1.0, std::floor(j.box[a] / (rl * (1.0 + 1e-4))));
-    const double groups = (double)j.n / 32.0 + ncell / 64.0 + 2.0;
-    return (double)j.n * 320.0 + groups * 32.0 * cap * 4.0 + ncell * 160.0 + 4.0 * 1024 * 1024;
+    const double bricks = ncell / 64.0 + 2.0;
+    const int group = small && o.list_layout == 0 && o.nbr_capacity == 0 ? dpd::group_for(j.n, bricks, cap, 1) : dpd::kGroup;
+    return (double)j.n * 320.0 + dpd::group_list_bytes(j.n, bricks, cap, group) + ncell * 160.0 + 4.0 * 1024 * 1024;
 }
 
 // Device bytes of a box in the ensemble: state, tags and indices (56 B per
@@ -534,8 +535,10 @@ dpd_status dpd_server_submit(dpd_server *S, const dpd_request *r, uint64_t *tick
         j.ens = j.ens_fit && S->opt.ensemble == 1;
     }
     j.est_ens_bytes = estimate_ensemble_bytes(j);
-    j.est_bytes = j.ens ? j.est_ens_bytes : estimate_bytes(j, S->opt.box_options);
+    j.est_bytes = j.ens ? j.est_ens_bytes : estimate_bytes(j, S->opt.box_options, false);
     if (j.est_bytes > S->budget) return fail_s(S, DPD_ERR_OOM, "box needs more device memory than the budget");
+    // accepted by what it cannot do without, counted by what it takes
+    if (!j.ens) j.est_bytes = std::min(estimate_bytes(j, S->opt.box_options, true), S->budget);
     {
         std::lock_guard<std::mutex> lk(S->m);
         if (S->stop) {

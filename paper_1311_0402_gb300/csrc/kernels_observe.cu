@@ -13,10 +13,11 @@ namespace {
 
 constexpr int kThreads = 256;
 
-// Error-free FP32 accumulation (FP64 arithmetic is scarce on this part):
-// s + c carries the exact running sum of a few dozen terms to about 2^-48
-// relative (Knuth's TwoSum for each addition; a square enters as its exact
-// two-term split hi + lo, hi = v v rounded, lo = fma(v, v, -hi)).
+// Compensated FP32 accumulation (FP64 arithmetic is scarce on this part):
+// Knuth's TwoSum for each addition, a square as its exact two-term split hi + lo,
+// hi = v v rounded, lo = fma(v, v, -hi).  Of the m terms one thread adds, s + c is
+// off by at most m^2 2^-48 of the sum of their magnitudes (the bound of Ogita,
+// Rump and Oishi).
 struct Sum2 {
     float s = 0.0f, c = 0.0f;
     // every operation rounded on its own: a contracted multiply-add would
@@ -35,30 +36,37 @@ struct Sum2 {
         c = __fadd_rn(c, fmaf(v, v, -hi));
     }
     __device__ __forceinline__ double value() const { return (double)s + (double)c; }
-    // lane 0: the sum over the warp, in a fixed order
-    __device__ __forceinline__ void warp_reduce()
-    {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float s2 = __shfl_down_sync(0xFFFFFFFFu, s, o), c2 = __shfl_down_sync(0xFFFFFFFFu, c, o);
-            add(s2);
-            c = __fadd_rn(c, c2);
-        }
-    }
 };
+
+// FP64 sums of four values over the warp, in a fixed order: lane 8 k returns the
+// sum of v[k].  Half the lanes hand two of their values over and keep the
+// other two, then a quarter one, so a lane makes 6 additions where four separate
+// trees make 20: FP64 additions are what limits this (one warp's take 16 cycles
+// of an SM).
+__device__ __forceinline__ double warp_sum4(const double (&v)[4], int lane)
+{
+    const bool hi2 = (lane & 16) != 0, hi1 = (lane & 8) != 0;
+    const double a = (hi2 ? v[2] : v[0]) + __shfl_xor_sync(0xFFFFFFFFu, hi2 ? v[0] : v[2], 16);
+    const double b = (hi2 ? v[3] : v[1]) + __shfl_xor_sync(0xFFFFFFFFu, hi2 ? v[1] : v[3], 16);
+    double x = (hi1 ? b : a) + __shfl_xor_sync(0xFFFFFFFFu, hi1 ? a : b, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
+    return x;
+}
 
 // Observables: sum v^2, sum v (3) over the particles, and the virial sum over
 // pairs inside r_c of r_ij . F^C_ij plus the bonds' share (Eq. 3 and Sec. 4.5).
 // The virial comes from the force evaluation that closed the last call (a force
 // evaluation, or the last step of a run): its positions are the current ones,
 // and the pair kernel left one partial per block in vir_part, summed here in a
-// fixed order.  The kinetic sums are exact to about 2^-48 per warp (Sum2), then
-// FP64.  Each block leaves its partials in red; the last one to finish adds all of
+// fixed order.  Each thread adds its particles as Sum2 (one particle up to
+// 155,648 of them); everything above a thread is FP64.  Each block leaves its
+// partials in red; the last one to finish adds all of
 // them in block order (whichever it is, the order is the same) and stores the
 // finished dpd_obs, nine 8-byte words: step, n, kinetic, temperature, virial,
 // pressure, momentum[3], with the divisors 3N - 3 and 3V passed in.  One launch
-// and FP32 warp sums where three launches reduced in FP64: 81,000 particles, a
-// step and its record each time: 91 to 78 us a step.
+// where there were three: 81,000 particles, a step and its record each time: 91
+// to 78 us a step.
 constexpr int kSums = 5;  // v^2, v (3), virial
 __global__ void __launch_bounds__(kThreads) k_observe(SimParams P, Ptrs D, double dof, double three_v)
 {
@@ -96,11 +104,9 @@ __global__ void __launch_bounds__(kThreads) k_observe(SimParams P, Ptrs D, doubl
         __syncthreads();
         return x;
     };
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        sums[k].warp_reduce();
-        if (lane == 0) sh[k][warp] = sums[k].value();
-    }
+    const double v4[4] = {sums[0].value(), sums[1].value(), sums[2].value(), sums[3].value()};
+    const double w4 = warp_sum4(v4, lane);
+    if ((lane & 7) == 0) sh[lane >> 3][warp] = w4;
     // most warps hold no virial partial
     if (__any_sync(0xFFFFFFFFu, first < nvir)) vir = warp_sum(vir);
     if (lane == 0) sh[4][warp] = vir;

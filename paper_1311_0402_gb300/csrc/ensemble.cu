@@ -55,7 +55,7 @@ struct dpd_ensemble {
     uint32_t *d_any_err = nullptr;
     int threads[kClasses] = {0, 0, 0, 0};
     int cluster[kClasses] = {0, 0, 0, 0};
-    bool tuned = false;
+    bool tuned[kClasses] = {};  // the size classes the autotuner has timed
     size_t limit = 0;
     bool failed = false;
     std::string err;
@@ -239,13 +239,13 @@ void fill_desc(EnsBox &d, const dpd_box_params *p, int64_t n, const int nc[3])
     d.key[3] = 0x85A308D3u;
 }
 
-// The shapes of the next launch: the autotuner's, else the options', else the
-// default for the boxes that run.
+// The shapes of the next launch, by size class: the autotuner's, else the
+// options', else the default for the boxes that run.
 void update_shapes(dpd_ensemble *e, const int (&count)[kClasses], const int64_t (&largest)[kClasses])
 {
-    if (e->tuned) return;
     const Shapes s = default_shapes(e->opt.newton3 != 0, count, largest);
     for (int c = 0; c < kClasses; ++c) {
+        if (e->tuned[c]) continue;
         e->threads[c] = e->opt.threads ? e->opt.threads : s.threads[c];
         e->cluster[c] = e->opt.cluster ? e->opt.cluster : s.cluster[c];
     }
@@ -925,8 +925,8 @@ dpd_status dpd_ensemble_tune(dpd_ensemble *e, int32_t steps, double *table)
         if (table) std::memcpy(table, tab, sizeof(tab));
         e->threads[cls] = best_t;
         e->cluster[cls] = best_c;
+        e->tuned[cls] = true;
     }
-    e->tuned = true;
     return ewait(e);
 }
 

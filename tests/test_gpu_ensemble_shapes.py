@@ -1,0 +1,39 @@
+"""Launch shapes of the ensemble."""
+import numpy as np
+import pytest
+
+import paper_1311_0402_gb300 as dpd
+import workloads
+from gpu_util import need_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+def _add(e, L, n, seed):
+    x, v = workloads.uniform_fluid((L, L, L), n, 1.0, seed)[:2]
+    return e.add((L, L, L), [[25.0]], 4.5, 1.0, 1.0, 1.0, 0.01, x, v, seed=seed)
+
+
+def test_a_class_without_boxes_at_tuning_keeps_the_rule():
+    """The tuner decides for the size classes it timed; boxes of another class
+    that come later run as in an ensemble that was never tuned."""
+    need_gpu()
+    e, fresh = dpd.Ensemble(), dpd.Ensemble()
+    _add(e, 5.0, 200, 1)
+    e.step(1)
+    e.sync()
+    e.tune(steps=2)
+    tuned = e.config()
+    k = int(np.flatnonzero(tuned[0])[0])
+    _add(e, 10.0, 3000, 2)
+    _add(fresh, 10.0, 3000, 2)
+    for h in (e, fresh):
+        h.step(1)
+        h.sync()
+    got, want = e.config(), fresh.config()
+    other = int(np.flatnonzero(want[0])[0])
+    assert other != k
+    assert (got[0][k], got[1][k]) == (tuned[0][k], tuned[1][k])
+    assert (got[0][other], got[1][other]) == (want[0][other], want[1][other])
+    e.close()
+    fresh.close()

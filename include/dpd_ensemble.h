@@ -131,7 +131,8 @@ dpd_status dpd_ensemble_info(dpd_ensemble *e, int32_t *nboxes, int64_t *nparticl
 dpd_status dpd_ensemble_tune(dpd_ensemble *e, int32_t steps, double *table);
 
 /* Per size class (0 = largest footprint .. 3), the threads per CTA and CTAs
- * per box the next launch uses (both 0 for a class without boxes). */
+ * per box that a step of all boxes uses (both 0 for a class without boxes; a
+ * step of some of them is launched for those). */
 dpd_status dpd_ensemble_config(dpd_ensemble *e, int32_t threads[4], int32_t cluster[4]);
 
 void dpd_ensemble_destroy(dpd_ensemble *e);

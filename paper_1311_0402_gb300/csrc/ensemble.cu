@@ -933,11 +933,16 @@ dpd_status dpd_ensemble_tune(dpd_ensemble *e, int32_t steps, double *table)
 dpd_status dpd_ensemble_config(dpd_ensemble *e, int32_t threads[4], int32_t cluster[4])
 {
     if (!e || !threads || !cluster) return efail(e, DPD_ERR_ARG, "null argument");
-    bool present[kClasses] = {false, false, false, false};
-    for (auto &kv : e->boxes) present[kv.second.cls] = true;
+    int count[kClasses] = {};
+    int64_t largest[kClasses] = {};
+    for (auto &kv : e->boxes) {
+        count[kv.second.cls] += 1;
+        largest[kv.second.cls] = std::max(largest[kv.second.cls], kv.second.n);
+    }
+    update_shapes(e, count, largest);
     for (int c = 0; c < kClasses; ++c) {
-        threads[c] = present[c] ? e->threads[c] : 0;
-        cluster[c] = present[c] ? e->cluster[c] : 0;
+        threads[c] = count[c] ? e->threads[c] : 0;
+        cluster[c] = count[c] ? e->cluster[c] : 0;
     }
     return DPD_OK;
 }

@@ -37,3 +37,16 @@ def test_a_class_without_boxes_at_tuning_keeps_the_rule():
     assert (got[0][other], got[1][other]) == (want[0][other], want[1][other])
     e.close()
     fresh.close()
+
+
+def test_config_reports_the_shapes_of_the_next_launch():
+    need_gpu()
+    e = dpd.Ensemble()
+    for k in range(3):
+        _add(e, 6.0, 600, k)
+    _add(e, 10.0, 3000, 9)
+    before = e.config()
+    e.step(1)
+    e.sync()
+    assert e.config() == before
+    e.close()

@@ -65,12 +65,13 @@ struct dpd_ensemble {
     cudaGraphExec_t graph = nullptr;
     std::vector<uint64_t> graph_key;
     int64_t graph_replays = 0;
-    // page-locked host memory that kernels write a box's state into, kept for
-    // the handle's life and as large as its largest read needs (a box has at
-    // most a few thousand particles)
-    double *mail = nullptr;
-    size_t mail_bytes = 0;
     int64_t graph_captures = 0;
+    // page-locked host memory that kernels write a box's state into, taken once
+    // and kept for the handle's life: taking it and giving it back can wait for
+    // the whole device.  `limit` bytes hold any box, which takes at least 53 B a
+    // particle of shared memory and 48 here.  (null when page-locked memory has
+    // run out: the reads then stage in device memory)
+    double *mail = nullptr;
 };
 
 namespace {
@@ -251,23 +252,6 @@ void update_shapes(dpd_ensemble *e, const int (&count)[kClasses], const int64_t 
     }
 }
 
-// e->mail of at least `bytes` (null when page-locked memory runs out: the
-// caller stages in device memory instead).
-double *ensure_mail(dpd_ensemble *e, size_t bytes)
-{
-    if (bytes <= e->mail_bytes) return e->mail;
-    if (e->mail) cudaFreeHost(e->mail);
-    e->mail = nullptr;
-    e->mail_bytes = 0;
-    if (cudaHostAlloc((void **)&e->mail, bytes, cudaHostAllocMapped) != cudaSuccess) {
-        cudaGetLastError();
-        e->mail = nullptr;
-        return nullptr;
-    }
-    e->mail_bytes = bytes;
-    return e->mail;
-}
-
 dpd_status ensure_desc(dpd_ensemble *e, size_t count)
 {
     if (count <= e->desc_cap) return DPD_OK;
@@ -368,6 +352,10 @@ dpd_status dpd_ensemble_create(dpd_ensemble **out, const dpd_ensemble_options *o
         cudaGetLastError();
         dpd_ensemble_destroy(e);
         return efail(nullptr, DPD_ERR_CUDA, "ensemble setup failed (no GPU, or kernel attributes refused)");
+    }
+    if (cudaHostAlloc((void **)&e->mail, e->limit, cudaHostAllocMapped) != cudaSuccess) {
+        cudaGetLastError();
+        e->mail = nullptr;
     }
     const int none[kClasses] = {};
     const int64_t zero[kClasses] = {};
@@ -678,7 +666,7 @@ dpd_status dpd_ensemble_get_state(dpd_ensemble *e, int32_t id, double *x, double
         // a box never stepped since its addition still needs its initial force
         // only for stepping; its state is the loaded one
         const size_t bytes = (size_t)b.n * 3 * sizeof(double);
-        if (double *m = ensure_mail(e, 2 * bytes)) {
+        if (double *m = e->mail) {
             // written straight into the page-locked block, one wait
             double *mv = m + 3 * (size_t)b.n;
             cudaError_t c = launch_export2(b.n, b.desc.pos, b.desc.vel, b.pid, x ? m : nullptr, v ? mv : nullptr, e->stream);

@@ -1,4 +1,4 @@
-"""Launch shapes of the ensemble."""
+"""Launch shapes of the ensemble, and reading states beside other work."""
 import numpy as np
 import pytest
 
@@ -49,4 +49,26 @@ def test_config_reports_the_shapes_of_the_next_launch():
     e.step(1)
     e.sync()
     assert e.config() == before
+    e.close()
+
+
+def test_reading_a_larger_box_does_not_wait_for_other_work():
+    """The block states are read through does not grow while other streams
+    run (page-locked memory taken or given back can wait for the device)."""
+    need_gpu()
+    e = dpd.Ensemble()
+    ids = [_add(e, 4.0 + k, 100 * (k + 1), k) for k in range(4)]
+    e.step(1)
+    e.sync()
+    e.state(ids[0])  # (the first launch of a kernel loads it, which waits)
+    x, v = workloads.uniform_fluid((40.0, 40.0, 40.0), 192000, 1.0, 3)[:2]
+    g = dpd.Sim((40.0, 40.0, 40.0), [[25.0]], 4.5, 1.0, 1.0, 1.0, 0.01)
+    g.set_state(x, v)
+    g.step(16)
+    g.step_async(4000)  # a quarter of a second
+    for i in ids:
+        assert np.isfinite(e.state(i)[0]).all()
+        assert not g.query()
+    g.sync()
+    g.close()
     e.close()

@@ -35,7 +35,12 @@ struct Sum2 {
         add(hi);
         c = __fadd_rn(c, fmaf(v, v, -hi));
     }
-    __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+    // by whole warps; a thread that added one term holds it in s alone
+    __device__ __forceinline__ double value() const
+    {
+        const double x = (double)s;
+        return __any_sync(0xFFFFFFFFu, c != 0.0f) ? x + (double)c : x;
+    }
 };
 
 // FP64 sums of four values over the warp, in a fixed order: lane 8 k returns the
@@ -125,11 +130,10 @@ __global__ void __launch_bounds__(kThreads) k_observe(SimParams P, Ptrs D, doubl
     for (int b = threadIdx.x; b < (int)gridDim.x; b += kThreads)
 #pragma unroll
         for (int k = 0; k < kSums; ++k) acc[k] += __ldcg(D.red + (size_t)b * 8 + k);
-#pragma unroll
-    for (int k = 0; k < kSums; ++k) {
-        const double x = warp_sum(acc[k]);
-        if (lane == 0) sh[k][warp] = x;
-    }
+    const double a4[4] = {acc[0], acc[1], acc[2], acc[3]};
+    const double t4 = warp_sum4(a4, lane), t5 = warp_sum(acc[4]);
+    if ((lane & 7) == 0) sh[lane >> 3][warp] = t4;
+    if (lane == 0) sh[4][warp] = t5;
     const double total = block_sums();
     if (threadIdx.x < kSums) sh[threadIdx.x][0] = total;
     __syncthreads();

@@ -156,6 +156,13 @@ size_t accepted_bytes(int64_t n, int ncell, bool lhalf)
     return l.total + ens_align16((size_t)n * 2) + 6144;
 }
 
+// The kernel packs places into kEnsPlaceBits bits; the shared memory of this
+// part (227 KB) ends near 4,300 particles.
+bool accepted(int64_t n, int ncell, bool lhalf, size_t limit)
+{
+    return n <= (int64_t)kEnsPlaceMask && accepted_bytes(n, ncell, lhalf) <= limit;
+}
+
 // Size class: how many CTAs of the box's footprint (256 threads) fit on one
 // SM -- 1 (class 0), 2, 3, or 4 and more (class 3).
 int class_of(int64_t n, int ncell, bool lhalf, size_t limit)
@@ -370,7 +377,7 @@ int32_t dpd_ensemble_fits(const dpd_box_params *p, int64_t n)
     if (!check_params(p, n, nc).empty()) return 0;
     const size_t limit = ensemble_smem_limit();
     if (limit == 0) return 0;
-    return accepted_bytes(n, nc[0] * nc[1] * nc[2], p->lambda == 0.5) <= limit ? 1 : 0;
+    return accepted(n, nc[0] * nc[1] * nc[2], p->lambda == 0.5, limit) ? 1 : 0;
 }
 
 dpd_status dpd_ensemble_add(dpd_ensemble *e, const dpd_box_params *p, int64_t n, const double *x, const double *v,
@@ -383,7 +390,7 @@ dpd_status dpd_ensemble_add(dpd_ensemble *e, const dpd_box_params *p, int64_t n,
     if (!why.empty()) return efail(e, DPD_ERR_ARG, why);
     const int ncell = nc[0] * nc[1] * nc[2];
     const bool lhalf = p->lambda == 0.5;
-    if (accepted_bytes(n, ncell, lhalf) > e->limit)
+    if (!accepted(n, ncell, lhalf, e->limit))
         return efail(e, DPD_ERR_ARG, "box does not fit one CTA's shared memory (" + std::to_string(n) + " particles)");
 
     EBox b;

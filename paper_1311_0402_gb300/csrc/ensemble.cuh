@@ -23,6 +23,8 @@ constexpr int kEnsWarpBytes = 32 * (4 * kEnsRanges + 2 * kEnsNotes);
 static_assert(kEnsWarpBytes >= 16 * kEnsQueue + 4 * kEnsCand, "the ring and the candidates share the scratch");
 constexpr int kEnsMaxCluster = 8;  // portable cluster size
 constexpr int kEnsMaxN = 65535;    // particle indices are 16-bit
+constexpr int kEnsPlaceBits = 13;  // places of the cell order and lengths of ranges, packed into a word with a shift
+constexpr uint32_t kEnsPlaceMask = (1u << kEnsPlaceBits) - 1u;
 
 // One box of a launch (filled by the host, read once per CTA).
 struct EnsBox {

@@ -350,9 +350,9 @@ __device__ __forceinline__ void ens_particle(const EnsBox &B, const EnsPtrs &S, 
     const int sub = lane % kEnsLanes;
     const int i = valid ? (int)S.idx[k] : 0;
     const float4 pi = S.pos[i], vi = S.u[i];
-    // the index ranges of this lane's rows: first place | length << 13 | shift << 26,
-    // the shift a base-3 code of (x, y, z), 0 none, 1 -L, 2 +L (a box that fits in
-    // shared memory has fewer than 2^13 particles)
+    // the index ranges of this lane's rows: first place | length << kEnsPlaceBits |
+    // shift << 2 kEnsPlaceBits, the shift a base-3 code of (x, y, z), 0 none, 1 -L, 2 +L
+    static_assert(2 * kEnsPlaceBits + 5 <= 32, "a shift code has 5 bits");
     int nr = 0;
     if (valid) {
         const int ncx = B.nc[0], ncy = B.nc[1], ncz = B.nc[2];
@@ -368,7 +368,7 @@ __device__ __forceinline__ void ens_particle(const EnsBox &B, const EnsPtrs &S, 
                 const int base = (z * ncy + y) * ncx;
                 auto add = [&](int c0, int c1, uint32_t code) {
                     const uint32_t b = S.start[base + c0], e = S.start[base + c1];
-                    if (e > b) ranges[nr++][lane] = b | ((e - b) << 13) | (code << 26);
+                    if (e > b) ranges[nr++][lane] = b | ((e - b) << kEnsPlaceBits) | (code << (2 * kEnsPlaceBits));
                 };
                 if (cx == 0) {
                     add(ncx - 1, ncx, sh + 1);
@@ -388,9 +388,9 @@ __device__ __forceinline__ void ens_particle(const EnsBox &B, const EnsPtrs &S, 
     int r = 0, noted = 0;
     auto next_range = [&]() {
         const uint32_t w = ranges[r++][lane];
-        q = w & 0x1FFFu;
-        qe = q + ((w >> 13) & 0x1FFFu);
-        const uint32_t code = w >> 26;
+        q = w & kEnsPlaceMask;
+        qe = q + ((w >> kEnsPlaceBits) & kEnsPlaceMask);
+        const uint32_t code = w >> (2 * kEnsPlaceBits);
         sx = shift_of(code % 3u, B.L[0]);
         sy = shift_of(code / 3u % 3u, B.L[1]);
         sz = shift_of(code / 9u, B.L[2]);

@@ -12,6 +12,7 @@
 // in one dpd_ensemble and advances every one of them a chunk per launch.
 #include "dpd_server.h"
 #include "dpd_internal.cuh"
+#include "serving.cuh"
 
 #include <algorithm>
 #include <atomic>
@@ -185,8 +186,7 @@ dpd_status start(dpd_server *S, Slot &sl)
                                sl.job.rc, sl.job.s, sl.job.dt, &o);
     if (st == DPD_OK) {
         std::lock_guard<std::mutex> lk(S->m);
-        const int64_t waiting = S->handle_active + (int64_t)S->pending.size();
-        dpd::expect_concurrent(sl.sim, (int)std::min<int64_t>(waiting, S->opt.max_active));
+        dpd::expect_concurrent(sl.sim, dpd::handles_expected(S->handle_active, S->pending, S->opt.max_active));
     }
     if (st != DPD_OK) {
         sl.sim = nullptr;

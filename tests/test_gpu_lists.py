@@ -93,3 +93,61 @@ def test_served_box_is_accepted_by_its_smallest_memory():
                 srv.submit(box, [[25.0]], 4.5, 1.0, 1.0, 1.0, 0.01, x, v, 20)
             assert e.value.status == 2
         srv.close()
+
+
+def test_a_box_of_more_cells_than_one_level_of_the_scan():
+    """Above 1,024 scan tiles (2.1 million cells) the tiles' totals are scanned
+    by a kernel of their own: a sparse box of 132^3 cells with a fluid in its last
+    corner, at load and after steps that rebuild."""
+    need_gpu()
+    L, corner, n = 172.0, 15.0, 14000
+    rng = np.random.default_rng(5)
+    x = rng.random((n, 3)) * L
+    m = 3 * int(corner ** 3)
+    x[:m] = L - corner * rng.random((m, 3))
+    x[m:m + 200, :2] *= 0.01  # and a column along one edge
+    v = rng.standard_normal((n, 3))
+    box = (L, L, L)
+    c = workloads.CONFIGS["fluid_small"]
+    g = dpd.Sim(box, c["a"], c["gamma"], c["kT"], c["rc"], c["s"], c["dt"], rebuild_every=2)
+    o = oracle.System(box, c["a"], c["gamma"], c["kT"], c["rc"], c["s"], c["dt"], cut_fp32=True)
+    g.set_state(x, v, step=1)
+    for _ in range(2):
+        x32, v32, step = g.state()
+        assert np.array_equal(g.neighbors(), oracle.pairs_fp32(x32, box, 1.3))
+        f, _ = o.forces(x32, v32, step=step)
+        assert force_error(g.forces(), f)[0] < FORCE_TOL
+        g.step(5)
+        g.build_neighbors()
+    g.close()
+
+
+# groups of 4, 8, 16 and 32; the row layout has lists and a pair kernel of its own
+@pytest.mark.parametrize("det", [0, 1])
+@pytest.mark.parametrize("n", [3000, 100000, 200001, 330000])
+def test_steps_that_rebuild_agree_with_the_row_layout(n, det):
+    """Six steps with a rebuild every second one (before the third and the
+    fifth).  The start is a jittered lattice (no near contacts).  A step rounds positions to a unit in the last
+    place of L (3.8e-6 up to L = 48), which moves a force by some 240 per unit
+    length and partner; a lost pair is a velocity error of 0.1 and more."""
+    need_gpu()
+    c = workloads.CONFIGS["fluid_small"]
+    k = int(np.ceil(n ** (1 / 3)))
+    L = (n / 3.0) ** (1 / 3)
+    rng = np.random.default_rng(n)
+    x = (np.stack(np.meshgrid(*[np.arange(k)] * 3, indexing="ij"), -1).reshape(-1, 3)[rng.permutation(k ** 3)[:n]]
+         + 0.5 + 0.2 * (rng.random((n, 3)) - 0.5)) * (L / k)
+    v = rng.standard_normal((n, 3))
+    out = []
+    for kw in (dict(deterministic=det), dict(deterministic=1, list_layout=1)):
+        g = dpd.Sim((L, L, L), c["a"], c["gamma"], c["kT"], c["rc"], c["s"], c["dt"], rebuild_every=2, **kw)
+        g.set_state(x, v)
+        r0 = g.info()["rebuilds"]
+        g.step(6)
+        assert g.info()["rebuilds"] >= r0 + 2
+        out.append(g.state())
+        g.close()
+    d = out[0][0] - out[1][0]
+    d -= L * np.round(d / L)
+    assert np.abs(d).max() < 5e-5
+    assert np.abs(out[0][1] - out[1][1]).max() < 2e-3

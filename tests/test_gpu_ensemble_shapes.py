@@ -2,9 +2,10 @@
 import numpy as np
 import pytest
 
+import oracle
 import paper_1311_0402_gb300 as dpd
 import workloads
-from gpu_util import need_gpu
+from gpu_util import force_error, need_gpu
 
 pytestmark = pytest.mark.gpu
 
@@ -71,4 +72,29 @@ def test_reading_a_larger_box_does_not_wait_for_other_work():
         assert not g.query()
     g.sync()
     g.close()
+    e.close()
+
+
+# more pairs than a lane notes; few particles; a box of 27 cells
+@pytest.mark.parametrize("n,L,shape", [(2000, 4.5, (512, 2)), (17, 3.5, (128, 4)), (90, 3.01, (256, 8))])
+def test_trajectories_of_sparse_and_dense_boxes(n, L, shape):
+    need_gpu()
+    box = (L, L + 0.3, L + 0.1)
+    x, v = workloads.uniform_fluid(box, n, 1.0, n)[:2]
+    a = [[2.0]]
+    e = dpd.Ensemble(threads=shape[0], cluster=shape[1])
+    i = e.add(box, a, 4.5, 1.0, 1.0, 0.5, 0.001, x, v, step=2, seed=7)
+    x32, v32, _ = e.state(i)
+    o = oracle.System(box, a, 4.5, 1.0, 1.0, 0.5, 0.001, seed=7, cut_fp32=True)
+    f0, _ = o.forces(x32, v32, step=2)
+    r = o.run(x32, v32, 3, step=2, f=f0)
+    e.step(3)
+    e.sync()
+    xg, vg, step = e.state(i)
+    assert step == r["step"] == 5
+    d = xg - r["x"]
+    d -= np.asarray(box) * np.round(d / np.asarray(box))
+    assert np.abs(d).max() < 1e-5
+    assert np.abs(vg - r["v"]).max() < 1e-3
+    assert force_error(e.forces(i), r["f"])[0] < 1e-3
     e.close()

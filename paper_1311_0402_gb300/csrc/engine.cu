@@ -221,6 +221,18 @@ void drop_graphs(dpd_sim *h)
     h->timed_graphs.clear();
 }
 
+// Whether a handle's kernels overlap their launches.  Not where the list builder
+// gathers from global memory (no bricks) or the rows are joined: the blocks of the
+// next kernel that wait on the SMs take their shared memory, presumably of the L1
+// cache that these kernels live on (us per step, overlapped / plain: a box of 2.7
+// x 100 x 100, 80,000 particles, 65 / 47, deterministic 124 / 76; no_reorder,
+// 100,000, 187 / 107; row layout 103 / 78).
+bool overlap_pays(const dpd_sim *h) { return h->P.use_bricks && h->P.list_layout == 0; }
+
+// Nor in a run of three handles side by side and more: the kernels that wait
+// early take the room the others' work would fill.
+bool overlaps(const dpd_sim *h) { return overlap_pays(h) && h->share < 3; }
+
 // Timing event on the stream; inside a graph capture it becomes an event
 // record node whose timestamp stays readable after the graph runs.
 // event record flags: external during stream capture (so the graph keeps
@@ -255,10 +267,6 @@ cudaError_t enqueue_steps_timed(dpd_sim *h, int64_t k)
     return e;
 }
 
-// Whether a handle's kernels overlap their launches.  Of three handles side by
-// side and more, the kernels that wait early take the room the others' work
-// would fill.
-bool overlaps(const dpd_sim *h) { return h->share < 3; }
 
 // Kernel sequence of k steps (starting and ending at a full-step state):
 // phase 1, then per step the rebuild chain (its kernels return at once unless
@@ -442,8 +450,8 @@ dpd_status rebuild_and_force(dpd_sim *h, bool grow_on_overflow)
         uint32_t one = 1u;
         CUDA_TRY(h, cudaMemcpyAsync(&h->D.ctl->rebuild, &one, sizeof(one), cudaMemcpyHostToDevice, h->stream));
         CUDA_TRY(h, cudaMemsetAsync(&h->D.ctl->err, 0, sizeof(uint32_t), h->stream));
-        CUDA_TRY(h, launch_rebuild(h->P, h->D, h->stream, h->n_scan_blocks, true));
-        CUDA_TRY(h, launch_force(h->P, h->D, kForceEval, false, h->stream, true));
+        CUDA_TRY(h, launch_rebuild(h->P, h->D, h->stream, h->n_scan_blocks, overlap_pays(h)));
+        CUDA_TRY(h, launch_force(h->P, h->D, kForceEval, false, h->stream, overlap_pays(h)));
         DevCtl c;
         dpd_status st = check_err(h, c);
         const int group = h->P.group;

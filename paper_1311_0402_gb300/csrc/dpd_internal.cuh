@@ -27,12 +27,15 @@
 #include <cuda_runtime.h>
 
 struct dpd_sim;
+struct dpd_ensemble;
 
 namespace dpd {
 
 // How many handles are expected to run side by side on the device (before the
 // first dpd_set_state; 1 unless called): each is then launched for its share.
 void expect_concurrent(dpd_sim *h, int handles);
+// Take the page-locked memory of an ensemble's state reads now, not at the first.
+void reserve_reads(dpd_ensemble *e);
 
 constexpr int kMaxSpecies = 8;
 constexpr int kMaxBonds = 6;          // bonds per particle

@@ -66,12 +66,14 @@ struct dpd_ensemble {
     std::vector<uint64_t> graph_key;
     int64_t graph_replays = 0;
     int64_t graph_captures = 0;
-    // page-locked host memory that kernels write a box's state into, taken once
-    // and kept for the handle's life: taking it and giving it back can wait for
-    // the whole device.  `limit` bytes hold any box, which takes at least 53 B a
-    // particle of shared memory and 48 here.  (null when page-locked memory has
-    // run out: the reads then stage in device memory)
+    // page-locked host memory that kernels write a box's state into, taken once,
+    // at the first read, and kept for the handle's life: taking it and giving it
+    // back can wait for the whole device, and takes 0.3 ms.  `limit` bytes hold any
+    // box, which takes at least 53 B a particle of shared memory and 48 here.
+    // (null when page-locked memory has run out: the reads then stage in device
+    // memory)
     double *mail = nullptr;
+    bool mail_asked = false;
 };
 
 namespace {
@@ -259,6 +261,17 @@ void update_shapes(dpd_ensemble *e, const int (&count)[kClasses], const int64_t 
     }
 }
 
+double *ensure_mail(dpd_ensemble *e)
+{
+    if (e->mail_asked) return e->mail;
+    e->mail_asked = true;
+    if (cudaHostAlloc((void **)&e->mail, e->limit, cudaHostAllocMapped) != cudaSuccess) {
+        cudaGetLastError();
+        e->mail = nullptr;
+    }
+    return e->mail;
+}
+
 dpd_status ensure_desc(dpd_ensemble *e, size_t count)
 {
     if (count <= e->desc_cap) return DPD_OK;
@@ -313,6 +326,8 @@ struct Group {
 
 }  // namespace
 
+void dpd::reserve_reads(dpd_ensemble *e) { ensure_mail(e); }
+
 extern "C" {
 
 void dpd_ensemble_default_options(dpd_ensemble_options *o)
@@ -359,10 +374,6 @@ dpd_status dpd_ensemble_create(dpd_ensemble **out, const dpd_ensemble_options *o
         cudaGetLastError();
         dpd_ensemble_destroy(e);
         return efail(nullptr, DPD_ERR_CUDA, "ensemble setup failed (no GPU, or kernel attributes refused)");
-    }
-    if (cudaHostAlloc((void **)&e->mail, e->limit, cudaHostAllocMapped) != cudaSuccess) {
-        cudaGetLastError();
-        e->mail = nullptr;
     }
     const int none[kClasses] = {};
     const int64_t zero[kClasses] = {};
@@ -673,7 +684,7 @@ dpd_status dpd_ensemble_get_state(dpd_ensemble *e, int32_t id, double *x, double
         // a box never stepped since its addition still needs its initial force
         // only for stepping; its state is the loaded one
         const size_t bytes = (size_t)b.n * 3 * sizeof(double);
-        if (double *m = e->mail) {
+        if (double *m = ensure_mail(e)) {
             // written straight into the page-locked block, one wait
             double *mv = m + 3 * (size_t)b.n;
             cudaError_t c = launch_export2(b.n, b.desc.pos, b.desc.vel, b.pid, x ? m : nullptr, v ? mv : nullptr, e->stream);

@@ -313,6 +313,7 @@ void ensemble_loop(dpd_server *S)
     };
     dpd_ensemble *E = nullptr;
     dpd_status est = dpd_ensemble_create(&E, nullptr);
+    if (est == DPD_OK) dpd::reserve_reads(E);
     std::string emsg = est == DPD_OK ? "" : std::string("ensemble: ") + dpd_ensemble_last_error(nullptr);
     std::vector<EJob> active;
     auto done_job = [&](EJob &ej, dpd_status st, const std::string &msg) {

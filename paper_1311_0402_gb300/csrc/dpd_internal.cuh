@@ -201,8 +201,13 @@ __device__ __forceinline__ void dependency_wait()
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// The same for a kernel that runs long where it does run: the next one is set up
+// when this one ends.  Set up earlier, its blocks would wait on the SMs all the
+// while, which costs nothing alone but takes the room of whatever runs beside.
+__device__ __forceinline__ void dependency_wait_long() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Launch k(args...); overlap: as a programmatic dependent of the kernel before
-// it on the stream (k then has to begin with dependency_wait()).
+// it on the stream (k then has to begin with dependency_wait() or _long()).
 template <typename... KArgs, typename... Args>
 cudaError_t launch_kernel(void (*k)(KArgs...), int grid, int block, size_t smem, cudaStream_t s, bool overlap, Args... args)
 {

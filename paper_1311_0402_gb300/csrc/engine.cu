@@ -222,11 +222,11 @@ void drop_graphs(dpd_sim *h)
 }
 
 // Whether a handle's kernels overlap their launches.  Not where the list builder
-// gathers from global memory (no bricks) or the rows are joined: the blocks of the
-// next kernel that wait on the SMs take their shared memory, presumably of the L1
-// cache that these kernels live on (us per step, overlapped / plain: a box of 2.7
-// x 100 x 100, 80,000 particles, 65 / 47, deterministic 124 / 76; no_reorder,
-// 100,000, 187 / 107; row layout 103 / 78).
+// gathers from global memory (no bricks) or the rows are joined: these kernels
+// live on the L1 cache, and where no SM falls idle between two kernels it
+// presumably keeps the share of shared memory that the pair kernel had (us per
+// step, overlapped / plain: a box of 2.7 x 100 x 100, 80,000 particles, 65 / 47,
+// deterministic 124 / 76; no_reorder, 100,000, 187 / 107; row layout 103 / 78).
 bool overlap_pays(const dpd_sim *h) { return h->P.use_bricks && h->P.list_layout == 0; }
 
 // Nor in a run of three handles side by side and more: the kernels that wait

@@ -826,7 +826,10 @@ __device__ __forceinline__ uint32_t build_cell(const SimParams &P, const float4 
 template <bool ATOMIC, bool ROWS>
 __global__ void __launch_bounds__(kBuildThreads, kBuildMinBlocks) k_nbuild_brick(SimParams P, Ptrs D)
 {
-    dependency_wait();
+    // (not releasing the pair kernel early: two handles of 250,000 particles side by
+    // side 125 us a step each when it did, 116 now, four of 81,000 95 and 88; one
+    // alone 71.2 and 71.2, 36.1 and 36.1)
+    dependency_wait_long();
     if (!D.ctl->rebuild) return;
     extern __shared__ float4 s_pos[];  // [P.brick_cap] staged halo positions
     __shared__ uint32_t s_off[kHaloCells + 1];

@@ -182,9 +182,11 @@ inline double group_list_bytes(int64_t n, double nbricks, double cap, int group)
 inline int group_for(int64_t n, double nbricks, double cap, int handles)
 {
     int group = kGroup;
-    while (group > kMinGroup && n < (int64_t)(kGroupsWanted / handles) * group &&
-           group_list_bytes(n, nbricks, cap, group / 2) <= kSmallGroupBytes)
+    while (group > kMinGroup) {
+        const int wanted = (group == kGroup ? kGroupsWanted : kGroupsWanted / 2) / handles;
+        if (n >= (int64_t)wanted * group || group_list_bytes(n, nbricks, cap, group / 2) > kSmallGroupBytes) break;
         group /= 2;
+    }
     return group;
 }
 

@@ -330,15 +330,18 @@ int group_count(const dpd_sim *h, int64_t n)
 
 // Particles per group list and builder blocks per brick.  A warp walks (and
 // builds) one group, so a box of few groups leaves most of the chip idle while
-// each warp works through a long list: groups are halved until there are
-// kGroupsWanted of them or they hold kMinGroup particles, and a brick's groups
-// are shared by enough blocks that each warp builds about one, up to
-// kBuildBlocksWanted blocks in all (each block stages the brick's halo anew).
+// each warp works through a long list: groups of 32 are halved while there are
+// fewer than kGroupsWanted of them, smaller ones while there are fewer than half
+// as many (16 particles below 320,000, 8 below 80,000, 4 below 40,000), and a
+// brick's groups are shared by enough blocks that each warp builds about one, up
+// to kBuildBlocksWanted blocks in all (each block stages the brick's halo anew).
 // us per step, groups of 32 / 16 / 8 / 4 with the best split of each:
 // 3,000 particles 46.6 / - / 26.8 / 24.0; 32,000 (rho = 4) 61.9 / 44.0 / 33.8 /
-// 33.5; 81,000 56.7 / 44.6 / 43.2 / 45.7; 207,000 73.5 / 68.4 / 69.6 / -;
-// 648,000 155.3 / 156.0 / - / -; 3,000,000 575 / 604 / - / -, and a split of
-// 2 there 591.  A fixed capacity keeps groups of 32, whose particles share it;
+// 33.5; 207,000 73.5 / 68.4 / 69.6 / -; 648,000 155.3 / 156.0 / - / -; 3,000,000
+// 575 / 604 / - / -, and a split of 2 there 591.  With fewer and overlapped
+// launches, one handle alone and four side by side: 45,000 - / - / 26.8, 55.9 /
+// 28.6, 66.2; 70,000 - / - / 33.1, 76.8 / 36.6, 89.1; 81,000 - / 35.6, 79.3 / 35.9,
+// 85.8; 155,000 - / 51.7, 138 / 53.2, 150; 250,000 72.8, 202 / 71.1, 209.  A fixed capacity keeps groups of 32, whose particles share it;
 // so do lists that would take more than kSmallGroupBytes (a box of thousands of
 // particles at hundreds of neighbours each).  Handles that run side by side each
 // want their share of the chip only (in deterministic mode the groups, which

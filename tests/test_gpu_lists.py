@@ -15,10 +15,10 @@ FORCE_TOL = 1e-4  # relative to the RMS force, max over particles/components
 
 
 # groups of 4, 8 and 16 particles.  Counted with the builder's rules for these
-# states: at the end a half list of 4 / 8 / 16 / 32 particles has up to 174 / 332
+# states: at the end a half list of 4 / 8 / 16 / 32 particles has up to 178 / 332
 # / 601 / 958 entries, where 32 x 32 = 1,024 is what 32 particles share at this
-# density; at the start, 39 / 61 / 90 / 149.
-@pytest.mark.parametrize("n,L", [(1500, 24.0), (100000, 97.0), (200000, 122.0)])
+# density; at the start, 36 / 61 / 91 / 144.
+@pytest.mark.parametrize("n,L", [(1500, 24.0), (60000, 82.0), (200000, 122.0)])
 def test_spots_that_condense_during_a_run_fit_the_lists(n, L):
     """24 spots of 45 free particles (no forces) contract to a seventh of their
     size while the handle steps: no list overflows, and every particle is
@@ -122,9 +122,10 @@ def test_a_box_of_more_cells_than_one_level_of_the_scan():
     g.close()
 
 
-# groups of 4, 8, 16 and 32; the row layout has lists and a pair kernel of its own
+# groups of 4 below 40,000 particles, 8 below 80,000, 16 below 320,000, else 32; the
+# row layout has lists and a pair kernel of its own
 @pytest.mark.parametrize("det", [0, 1])
-@pytest.mark.parametrize("n", [3000, 100000, 200001, 330000])
+@pytest.mark.parametrize("n", [3000, 39999, 40000, 100000, 200001, 330000])
 def test_steps_that_rebuild_agree_with_the_row_layout(n, det):
     """Six steps with a rebuild every second one (before the third and the
     fifth).  The start is a jittered lattice (no near contacts).  A step rounds positions to a unit in the last

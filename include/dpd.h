@@ -46,7 +46,7 @@ typedef enum {
                                  DPD_TEST_FAIL_ALLOC=1 makes every device allocation
                                  of a handle fail this way) */
     DPD_ERR_CUDA = 3,         /* a CUDA call failed (latched) */
-    DPD_ERR_NBR_OVERFLOW = 4, /* a group of 32 particles had more pairs than its list holds */
+    DPD_ERR_NBR_OVERFLOW = 4, /* a group of particles had more pairs than its list holds */
     DPD_ERR_NONFINITE = 5,    /* a force or position became NaN / Inf */
     DPD_ERR_TIMEOUT = 6,      /* the GPU did not finish within the wait limit */
     DPD_ERR_STATE = 7         /* call order: e.g. dpd_step before dpd_set_state */

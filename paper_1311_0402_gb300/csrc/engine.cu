@@ -341,10 +341,11 @@ int group_count(const dpd_sim *h, int64_t n)
 // 575 / 604 / - / -, and a split of 2 there 591.  With fewer and overlapped
 // launches, one handle alone and four side by side: 45,000 - / - / 26.8, 55.9 /
 // 28.6, 66.2; 70,000 - / - / 33.1, 76.8 / 36.6, 89.1; 81,000 - / 35.6, 79.3 / 35.9,
-// 85.8; 155,000 - / 51.7, 138 / 53.2, 150; 250,000 72.8, 202 / 71.1, 209.  A fixed capacity keeps groups of 32, whose particles share it;
-// so do lists that would take more than kSmallGroupBytes (a box of thousands of
-// particles at hundreds of neighbours each).  Handles that run side by side each
-// want their share of the chip only (in deterministic mode the groups, which
+// 85.8; 155,000 - / 51.7, 138 / 53.2, 150; 250,000 72.8, 202 / 71.1, 209.
+// A fixed capacity keeps groups of 32, whose particles share it; so do lists that
+// would take more than kSmallGroupBytes (a box of thousands of particles at
+// hundreds of neighbours each).  Handles that run side by side and are known to
+// each want their share of the chip only (in deterministic mode the groups, which
 // order the sums, stay those of a handle alone).
 void set_group(dpd_sim *h, int64_t n, int group)
 {

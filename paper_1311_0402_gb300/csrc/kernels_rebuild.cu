@@ -19,7 +19,7 @@
 //              the other buffer set
 //   k_sort_small  all of the above in one launch, for small boxes
 //   k_nbuild_brick / k_nbuild
-//              packed neighbour lists of groups of 32 particles, hits
+//              packed neighbour lists of groups of 4 to 32 particles, hits
 //              compacted by warp ballots as in the paper's builder (Sec. 3.3);
 //              the list order depends only on the positions
 #include "dpd_internal.cuh"
@@ -538,9 +538,9 @@ __global__ void k_nbuild(SimParams P, Ptrs D)
     if (lane == 0 && local_max) atomicMax(&D.ctl->max_nnb, local_max);
 }
 
-// Brick builder: one CTA per brick (see brick.cuh).  The CTA stages the
+// Brick builder: P.brick_split CTAs per brick (see brick.cuh).  Each stages the
 // positions of the brick's halo in shared memory with bulk (TMA) copies;
-// its warps take the brick's particles in groups of 32 and build each
+// their warps take the brick's particles in groups of P.group and build each
 // group cell by cell.  For a cell C the warp lays out one candidate
 // sequence: C's own particles (index order), then the particles of the
 // stencil cells it needs -- in Newton-3 mode those of higher rank than C,
@@ -551,7 +551,7 @@ __global__ void k_nbuild(SimParams P, Ptrs D)
 // the group in C, all 32 lanes test 32 consecutive candidates per
 // iteration, the owner's position broadcast from shared memory, and append
 // the hits with a ballot.  No lane diverges and the list order is fixed by
-// the positions.  The groups of brick b get the ids lo/32 + ord(b) onwards,
+// the positions.  The groups of brick b get the ids lo / P.group + ord(b) onwards,
 // where ord is the brick's position in rank order: unique ids with no count
 // pass; the ids a brick leaves unused (at most one or two) get empty
 // descriptors.  A brick whose halo exceeds the staging buffer reads

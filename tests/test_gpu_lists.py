@@ -74,6 +74,37 @@ def test_a_spot_too_dense_for_small_groups_at_load(det):
     g.close()
 
 
+def test_a_list_that_cannot_grow_leaves_no_state(monkeypatch):
+    """A rebuild whose lists have to grow and get no memory (refused on the host)
+    leaves the handle without a state, not with the lists it gave back; the next
+    load is an ordinary one."""
+    need_gpu()
+    box, n = (16.0, 16.0, 16.0), 1000
+    x, v = workloads.uniform_fluid(box, n, 0.0, 4)[:2]
+    c = np.array([8.3, 8.3, 8.3])
+    u = 0.9 * (x[:60] / 16.0 - 0.5) * 4.0
+    x[:60], v[:60] = c + u, -0.85 * u  # a spot that contracts within a time unit
+    g = dpd.Sim(box, [[0.0]], 0.0, 0.0, 1.0, 1.0, 0.01)
+    g.set_state(x, v)
+    assert g.info()["nbr_capacity"] == 32
+    g.step(100)
+    monkeypatch.setenv("DPD_TEST_FAIL_ALLOC", "1")
+    with pytest.raises(dpd.DPDError) as e:
+        g.build_neighbors()
+    assert e.value.status == 2  # DPD_ERR_OOM
+    monkeypatch.delenv("DPD_TEST_FAIL_ALLOC")
+    with pytest.raises(dpd.DPDError) as e:
+        g.step(1)
+    assert e.value.status == 7  # DPD_ERR_STATE
+    g.set_state(x, v)
+    g.step(100)
+    g.build_neighbors()
+    assert g.info()["nbr_capacity"] > 32
+    x32, _, _ = g.state()
+    assert np.array_equal(g.neighbors(), oracle.pairs_fp32(x32, box, 1.3))
+    g.close()
+
+
 def test_served_box_is_accepted_by_its_smallest_memory():
     """A budget that holds the box with lists of 32 particles a group is enough,
     and what is counted stays within it."""
